@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "step2d_tile.cuh"
 #include "wave_internal.cuh"
 
 using namespace wave;
@@ -478,6 +479,176 @@ static cudaError_t run_step(const wave_model_s* m, const StepArgs& a, cudaStream
   return err;
 }
 
+// ---- several 2D steps per launch (step2d_tile.cu) ----------------------------
+// Buffers of a time loop that advances several levels per launch: two pairs of
+// levels (a launch reads one and writes the other) and the per-region receiver
+// lists.
+struct TileWs {
+  bool on = false;
+  Tile2DPlan plan;
+  float* u[2][2];    // [pair][u^{n-1}, u^n]
+  int *count, *ptr, *cursor;
+  void* ent;
+  int64_t entries = 0;
+};
+
+// Region split for the model's 2D grid: rows per warp (2 or 4; 16 warps) and
+// steps per launch S that minimise the modelled time of a step,
+//   (launch + waves * (edge + S * step)) / S,
+// over 152 CTAs a wave.  The figures are fits to measured gradient calls (128^2
+// and 251^2 order 2, 2048^2 order 8, 6001 x 8003 order 4 on GB300): about 5 us
+// for a region's loads, lists and stores, 1 us a launch, and per step
+// rb (0.13 + 0.04 r) us but at least 0.5.  A small grid thus takes deep
+// regions (the halo work runs on SMs that would idle), a large one shallow ones.
+// Grids below 128 cells in x or 16 in y, above 2^29 cells (the second pair of
+// levels costs 2 grids) and the other storage types keep one step per launch.
+static bool tile2d_plan(const wave_model_s* m, int32_t maxrec, Tile2DPlan* out, int64_t* entries) {
+  const Geom& g = m->g;
+  if (m->d.ndim != 2 || m->d.physics != WAVE_VELOCITY || m->d.storage != WAVE_F32) return false;
+  if (g.nx < kStrip || g.ny < 16 || g.cells > ((int64_t)1 << 29)) return false;
+  const int nx = (int)g.nx, ny = (int)g.ny, r = g.r;
+  double best = 0.0;
+  bool found = false;
+  for (int rb = 2; rb <= 4; rb += 2) {
+    const int rh = std::min(rb * 16, ny / rb * rb);
+    const double step_us = std::max(0.5, rb * (0.13 + 0.04 * r));
+    for (int h = 4; h <= 56; h += 4) {   // multiples of 4: owned ranges keep whole quads
+      if (h % r) continue;
+      Tile2DPlan p;
+      p.rb = rb;
+      p.rh = rh;
+      p.steps = h / r;
+      p.h = h;
+      p.outx = kStrip - 2 * h;
+      p.outy = rh - 2 * h;
+      if ((nx > kStrip && p.outx < 1) || (ny > rh && p.outy < 1)) continue;
+      p.nkx = nx == kStrip ? 1 : 1 + (nx - kStrip + p.outx - 1) / p.outx;
+      p.nky = ny == rh ? 1 : 1 + (ny - rh + p.outy - 1) / p.outy;
+      if (p.nkx == 1) p.outx = kStrip;
+      if (p.nky == 1) p.outy = rh;
+      if (p.nky > 65535) continue;
+      const double waves = ceil((double)p.nkx * p.nky / 152.0);
+      const double t = (1.0 + waves * (5.0 + p.steps * step_us)) / p.steps;
+      if (!found || t < best) {
+        best = t;
+        *out = p;
+        found = true;
+      }
+    }
+  }
+  if (!found) return false;
+  // a cell lies in at most (w - 1) / out + 1 of the evenly placed regions of an axis, and the last one
+  const int64_t bx = std::min(out->nkx, (kStrip - 1) / out->outx + 2);
+  const int64_t by = std::min(out->nky, (out->rh - 1) / out->outy + 2);
+  *entries = bx * by * std::max(maxrec, 1);
+  return *entries < ((int64_t)1 << 30);
+}
+
+static void carve_tile(Carve& c, const wave_model_s* m, int32_t maxrec, void* u0, void* u1, TileWs* t) {
+  t->on = tile2d_plan(m, maxrec, &t->plan, &t->entries);
+  if (!t->on) return;
+  const size_t n = (size_t)t->plan.nkx * t->plan.nky;
+  t->u[0][0] = static_cast<float*>(u0);
+  t->u[0][1] = static_cast<float*>(u1);
+  t->u[1][0] = c.take<float>(m->g.cells);
+  t->u[1][1] = c.take<float>(m->g.cells);
+  t->count = c.take<int>(n);
+  t->cursor = c.take<int>(n);
+  t->ptr = c.take<int>(n + 1);
+  t->ent = c.take<int2>(t->entries);
+}
+
+static Tile2DArgs tile_args(const wave_model_s* m, const TileWs& t, const wave_shot& sh) {
+  Tile2DArgs a;
+  memset(&a, 0, sizeof(a));
+  a.g = m->g;
+  a.plan = t.plan;
+  a.coef = m->coef;
+  a.h2 = (float)(m->d.h * m->d.h);
+  a.nrec = sh.nrec;
+  a.tptr = t.ptr;
+  a.tent = static_cast<const int2*>(t.ent);
+  a.sx = (int)(sh.src_cell % m->g.nx);
+  a.sy = (int)(sh.src_cell / m->g.nx);
+  a.wavelet = sh.wavelet_dev;
+  return a;
+}
+
+// One launch of a.nsteps steps; the timing and metrics count every step.
+static cudaError_t run_tile(const wave_model_s* m, const Tile2DArgs& a, cudaStream_t s) {
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (g_timing.on) {
+    while (g_timing.ev.size() < g_timing.used + 2) {
+      cudaEvent_t e;
+      cudaError_t err = cudaEventCreate(&e);
+      if (err != cudaSuccess) return err;
+      g_timing.ev.push_back(e);
+    }
+    e0 = g_timing.ev[g_timing.used];
+    e1 = g_timing.ev[g_timing.used + 1];
+    g_timing.used += 2;
+    cudaError_t err = record_event(e0, s);
+    if (err != cudaSuccess) return err;
+  }
+  cudaError_t err = launch_tile2d_velocity(a, m->d.order, s);
+  if (err != cudaSuccess) return err;
+  const double cells = (double)(m->g.nx * m->g.ny * m->g.nz);
+  const int acc_steps = a.acc ? std::max(0, std::min(a.nsteps, a.mass_hi) - a.mass_lo) : 0;
+  const double bytes = cells * (16.0 * a.nsteps + (a.comp ? 16.0 : 8.0) * acc_steps);
+  if (g_timing.on) {
+    err = record_event(e1, s);
+    g_timing.bytes += bytes;
+    g_timing.launches += a.nsteps;
+  }
+  if (m->met.on) {
+    m->met.bytes += bytes;
+    m->met.launches += a.nsteps;
+  }
+  return err;
+}
+
+// Levels u^1.. of a shot forward to u^{N+1} from pair `at` (u^0, u^1);
+// records levels 1..N into what `a` names.  acc != null: -K(u,u) increments of
+// steps 1..N-1.  Returns the pair that holds (u^N, u^{N+1}) in *at.
+static cudaError_t tile_forward(const wave_model_s* m, const TileWs& t, Tile2DArgs a, int N, int* at, cudaStream_t s) {
+  a.acc_scale = 1.f;
+  a.dlevel = 1;
+  for (int n = 1; n <= N; n += t.plan.steps) {
+    a.nsteps = std::min(t.plan.steps, N - n + 1);
+    a.level0 = n;
+    a.mass_hi = N - n;
+    a.prev = t.u[*at][0];
+    a.cur = t.u[*at][1];
+    *at ^= 1;
+    a.oprev = t.u[*at][0];
+    a.ocur = t.u[*at][1];
+    cudaError_t e = run_tile(m, a, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// The superposed pass j = N..1 from pair `at` holding (u^N, u^{N+1}).
+static cudaError_t tile_superposed(const wave_model_s* m, const TileWs& t, Tile2DArgs a, int N, int at, cudaStream_t s) {
+  a.acc_scale = -1.f;
+  a.dlevel = -1;
+  a.prev = t.u[at][1];
+  a.cur = t.u[at][0];
+  for (int j = N; j >= 1; j -= t.plan.steps) {
+    a.nsteps = std::min(t.plan.steps, j);
+    a.level0 = j;
+    a.mass_hi = a.nsteps;
+    at ^= 1;
+    a.oprev = t.u[at][0];
+    a.ocur = t.u[at][1];
+    cudaError_t e = run_tile(m, a, s);
+    if (e != cudaSuccess) return e;
+    a.prev = a.oprev;
+    a.cur = a.ocur;
+  }
+  return cudaSuccess;
+}
+
 static cudaError_t run_batched(const wave_model_s* m, const BatchArgs& b, cudaStream_t s) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (g_timing.on) {
@@ -608,13 +779,14 @@ extern "C" wave_status wave_step(wave_model m, int32_t nfields, const void* cons
 // forward
 // ---------------------------------------------------------------------------
 static void carve_forward(Carve& c, const wave_model_s* m, const wave_shot* shots, int32_t nshots, void** u0,
-                          void** u1, int64_t** recp) {
+                          void** u1, int64_t** recp, TileWs* tw) {
   int32_t maxrec = 1;
   for (int s = 0; s < nshots; ++s) maxrec = std::max(maxrec, shots[s].nrec);
   const size_t eb = storage_bytes(m->d.storage);
   *u0 = c.take_bytes(m->g.cells * eb);
   *u1 = c.take_bytes(m->g.cells * eb);
   *recp = c.take<int64_t>(maxrec);
+  carve_tile(c, m, maxrec, *u0, *u1, tw);
 }
 
 extern "C" wave_status wave_forward_workspace_size(wave_model m, const wave_shot* shots, int32_t nshots,
@@ -625,7 +797,8 @@ extern "C" wave_status wave_forward_workspace_size(wave_model m, const wave_shot
   Carve c(nullptr);
   void *u0, *u1;
   int64_t* recp;
-  carve_forward(c, m, shots, nshots, &u0, &u1, &recp);
+  TileWs tw;
+  carve_forward(c, m, shots, nshots, &u0, &u1, &recp, &tw);
   *bytes = c.off;
   return WAVE_OK;
 }
@@ -645,7 +818,8 @@ extern "C" wave_status wave_forward(wave_model m, const wave_shot* shots, int32_
   Carve c(ws);
   void *ua, *ub;
   int64_t* recp;
-  carve_forward(c, m, shots, nshots, &ua, &ub, &recp);
+  TileWs tw;
+  carve_forward(c, m, shots, nshots, &ua, &ub, &recp, &tw);
   const int64_t ncells = g.nx * g.ny * g.nz;
   for (int si = 0; si < nshots; ++si) {
     const wave_shot& sh = shots[si];
@@ -664,6 +838,20 @@ extern "C" wave_status wave_forward(wave_model m, const wave_shot* shots, int32_
     sp.gsrc = ua;
     sp.glevel = 0;
     CUDA_TRY(launch_sparse(sp, stor, s));
+    if (tw.on) {
+      Tile2DArgs a = tile_args(m, tw, sh);
+      a.traces = sh.traces_dev;
+      a.tr_ld = N + 1;
+      CUDA_TRY(launch_tile2d_lists(tw.plan, g, recp, sh.nrec, tw.count, tw.ptr, tw.cursor, tw.ent, s));
+      CUDA_TRY(launch_tile2d_skipped(recp, sh.nrec, 1, N, nullptr, sh.traces_dev, N + 1, s));
+      int at = 0;
+      CUDA_TRY(tile_forward(m, tw, a, N, &at, s));
+      if (final_dev && si == nshots - 1) {
+        CUDA_TRY(launch_pitched_to_dense(g, tw.u[at][0], final_dev, stor, s));
+        CUDA_TRY(launch_pitched_to_dense(g, tw.u[at][1], final_dev + ncells, stor, s));
+      }
+      continue;
+    }
     sp.gsrc = ub;
     sp.glevel = 1;
     sp.dst = ua;
@@ -707,6 +895,7 @@ struct GradWs {
   int64_t* recp;
   double* parts;
   double* scal;  // [0] k, [1] psi2, [2] e2, [3] C (no caller buffer), [4] sum grad^2, [6] C copy
+  TileWs tile;
 };
 
 static void carve_gradient(Carve& c, const wave_model_s* m, const wave_shot* shots, int32_t nshots, int mode,
@@ -729,6 +918,7 @@ static void carve_gradient(Carve& c, const wave_model_s* m, const wave_shot* sho
   w->recp = c.take<int64_t>(maxrec);
   w->parts = c.take<double>(1024);
   w->scal = c.take<double>(8);
+  if (!two) carve_tile(c, m, maxrec, w->u0, w->u1, &w->tile);
 }
 
 static wave_status validate_opts(const wave_model_s* m, const wave_gradient_opts* o) {
@@ -1188,17 +1378,34 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
     sp.gsrc = w.u0;
     sp.glevel = 0;
     CUDA_TRY(launch_sparse(sp, stor, s));
-    sp.gsrc = w.u1;
-    sp.glevel = 1;
-    sp.dst = w.u0;
-    sp.src_p = pitched_cell(g, sh.src_cell);
-    sp.wavelet = sh.wavelet_dev;
-    sp.ilevel = 1;
-    CUDA_TRY(launch_sparse(sp, stor, s));
+    const bool tile = w.tile.on;
+    int at = 0;   // level pair of the several-steps-per-launch path
+    Tile2DArgs ta;
+    if (tile) {
+      ta = tile_args(m, w.tile, sh);
+      ta.acc = w.acc;
+      ta.comp = w.comp;
+      CUDA_TRY(launch_tile2d_lists(w.tile.plan, g, w.recp, sh.nrec, w.tile.count, w.tile.ptr, w.tile.cursor,
+                                   w.tile.ent, s));
+      CUDA_TRY(launch_tile2d_skipped(w.recp, sh.nrec, 1, N, w.resid, nullptr, 0, s));
+      Tile2DArgs f = ta;
+      f.resid = w.resid;
+      f.observed = sh.observed_dev;
+      f.obs_ld = N + 1;
+      CUDA_TRY(tile_forward(m, w.tile, f, N, &at, s));
+    } else {
+      sp.gsrc = w.u1;
+      sp.glevel = 1;
+      sp.dst = w.u0;
+      sp.src_p = pitched_cell(g, sh.src_cell);
+      sp.wavelet = sh.wavelet_dev;
+      sp.ilevel = 1;
+      CUDA_TRY(launch_sparse(sp, stor, s));
+    }
     // ---- forward: propagate, adjoint source, -K(u,u) ------------------
     void* prev = w.u0;
     void* cur = w.u1;
-    for (int n = 1; n <= N; ++n) {
+    for (int n = 1; n <= N && !tile; ++n) {
       StepArgs a = step_args(m, cur, prev);
       a.acc = w.acc;
       a.comp = w.comp;
@@ -1348,6 +1555,13 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
         }
         for (int f = 0; f < 2; ++f) std::swap(fc[f], fn[f]);
       }
+      continue;
+    }
+    if (tile) {
+      ta.resid_in = w.resid;
+      ta.k_dev = kd;
+      ta.weight = (float)wgt;
+      CUDA_TRY(tile_superposed(m, w.tile, ta, N, at, s));
       continue;
     }
     // ---- superposed pass: u^s from (u^{N+1}, u^N), +K(u^s,u^s) ----------

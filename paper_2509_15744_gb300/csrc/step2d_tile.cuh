@@ -1,0 +1,70 @@
+// Several 2D leapfrog steps per launch (step2d_tile.cu): the split of the
+// domain into regions and the launch arguments.
+#pragma once
+
+#include "wave_internal.cuh"
+
+namespace wave {
+
+// Regions of 128 x rh cells, outx x outy of them owned inside the domain;
+// consecutive regions overlap by 2 h with h = r * steps.  rb: rows per warp.
+struct Tile2DPlan {
+  int rb, rh, steps, h;
+  int outx, outy;
+  int nkx, nky;
+};
+
+// First cell of region k along an axis of n cells cut into nk regions of w
+// cells: every `out` cells, the last one ends at n.
+__host__ __device__ __forceinline__ int tile_start(int k, int nk, int out, int n, int w) {
+  return k < nk - 1 ? k * out : n - w;
+}
+// Owned cells [lo, hi): from where the previous region's stop to h before the
+// region's own end; the first from 0, the last to n.
+__host__ __device__ __forceinline__ int tile_own_lo(int k, int out, int w, int h) {
+  return k == 0 ? 0 : (k - 1) * out + w - h;
+}
+__host__ __device__ __forceinline__ int tile_own_hi(int k, int nk, int out, int n, int w, int h) {
+  return k == nk - 1 ? n : k * out + w - h;
+}
+
+struct Tile2DArgs {
+  Geom g;
+  Tile2DPlan plan;
+  const float* prev;      // level n-1
+  const float* cur;       // level n
+  float* oprev;           // level n+nsteps-1 (other buffers than prev, cur)
+  float* ocur;            // level n+nsteps
+  const float* coef;
+  float* acc;             // sensitivity accumulator (nullable), updated in place
+  float* comp;            // Kahan compensation (nullable)
+  float acc_scale;        // +1 or -1
+  int nsteps;             // <= plan.steps
+  int mass_lo, mass_hi;   // steps of the launch that accumulate
+  int level0, dlevel;     // recorded / injected level of the first step, and its change per step
+  // receivers (lists per region: entries ptr[t] .. ptr[t+1])
+  int nrec;
+  const int* tptr;
+  const int2* tent;       // {row * 128 + column in the region | owned << 31, receiver}
+  float* resid;           // record u - d, time-major (nullable)
+  const float* observed;
+  int64_t obs_ld;
+  float* traces;          // record u, receiver-major (nullable)
+  int64_t tr_ld;
+  const float* resid_in;  // inject -k w e, time-major residuals (nullable)
+  const double* k_dev;
+  float weight;
+  // source
+  int sx, sy;
+  const float* wavelet;   // nullable
+  float h2;
+};
+
+int tile2d_smem(const Tile2DPlan& p);
+cudaError_t launch_tile2d_velocity(const Tile2DArgs& a, int order, cudaStream_t s);
+cudaError_t launch_tile2d_lists(const Tile2DPlan& p, const Geom& g, const int64_t* rec_p, int nrec, int* count,
+                                int* ptr, int* cursor, void* ent, cudaStream_t s);
+cudaError_t launch_tile2d_skipped(const int64_t* rec_p, int nrec, int lo, int hi, float* resid, float* traces,
+                                  int64_t tr_ld, cudaStream_t s);
+
+}  // namespace wave

@@ -1,0 +1,84 @@
+"""Several 2D steps per launch (csrc/step2d_tile.cu): regions of the grid that
+overlap by the steps' halo.
+
+The forward from given levels and no force must give the bits of the same
+number of single steps (`Model.step`, the one-step kernel) at every edge of
+the split: grids one region wide or high, one cell more than a region, last
+regions at unaligned offsets, step counts that leave a remainder.  Gradients
+with receivers in several regions, duplicated receivers and receivers outside
+the grid are held to the oracle at the parity bars of the other tests (traces
+1e-4, sensitivity 1e-3 at the same k).
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from _gpu import gpu_model, gpu_shots
+from _problems import make_problem, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(16, 128), (17, 129), (64, 128), (65, 131), (130, 257), (203, 383)]
+
+
+@pytest.fixture(scope="module")
+def W():
+    import __graft_entry__ as ge
+    ge.build()
+    from paper_2509_15744_gb300 import wave
+    return wave
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("order,bc,nt", [(2, "dirichlet", 61), (4, "neumann", 33), (6, "dirichlet", 23),
+                                         (8, "neumann", 19), (8, "dirichlet", 1)])
+def test_forward_has_the_bits_of_single_steps(W, shape, order, bc, nt):
+    rng = np.random.default_rng(7)
+    v = torch.from_numpy(rng.uniform(1500, 3000, shape).astype(np.float32)).cuda()
+    m = W.Model(v, 10.0, O.cfl_dt(10.0, 3000.0, 2, order, 0.5), order, "velocity", bc)
+    init = torch.from_numpy(rng.standard_normal((2,) + shape).astype(np.float32)).cuda()
+    none = torch.zeros(0, dtype=torch.int64, device="cuda")
+    shot = W.Shot(0, torch.zeros(nt + 1, device="cuda"), none)
+    _, final = m.forward([shot], init=init, return_final=True)
+    a, b = (torch.zeros(m.pitched_shape(), device="cuda") for _ in range(2))
+    a[:, :shape[1]], b[:, :shape[1]] = init[0], init[1]
+    for _ in range(nt):
+        m.step([b], [a])
+        a, b = b, a
+    torch.cuda.synchronize()
+    assert torch.equal(final[0], a[:, :shape[1]])
+    assert torch.equal(final[1], b[:, :shape[1]])
+
+
+@pytest.mark.parametrize("shape,order,bc,kahan,objective", [
+    ((65, 131), 2, "neumann", False, "l2"), ((130, 257), 4, "dirichlet", True, "l2"),
+    ((77, 150), 8, "dirichlet", False, "patch"), ((40, 300), 6, "neumann", True, "patch")])
+def test_gradient_matches_the_oracle(W, shape, order, bc, kahan, objective):
+    ny, nx = shape
+    if objective == "patch":   # dense: more entries than threads in the regions that hold it
+        yy, xx = np.meshgrid(np.arange(8, ny - 8), np.arange(20, 100), indexing="ij")
+        kw = dict(patch=(yy * nx + xx).ravel(), src=(ny // 2) * nx + 12)
+    else:                      # on the edges, twice in one cell, on the source
+        rec = np.unique(np.concatenate([np.arange(0, nx, 3), (ny - 1) * nx + np.arange(0, nx, 3),
+                                        np.arange(0, ny * nx, nx), np.arange(nx - 1, ny * nx, nx)]))
+        kw = dict(rec=np.concatenate([rec, rec[:5], [2 * nx + 30]]), src=2 * nx + 30)
+    prob = make_problem(shape, order, bc, nt=60, seed=5, objective=objective, **kw)
+    m = gpu_model(W, prob, kahan=kahan)
+    g, c, k = m.gradient(gpu_shots(W, prob), objective=objective)
+    ref = O.superposition_gradient(prob.medium(), prob.oracle_shots(), prob.nt[0], float(k.item()))
+    assert rel_l2(g.cpu().numpy(), ref["K_tilde"]) < 1e-3
+    assert abs(float(c.item()) - ref["C"]) < 1e-5 * abs(ref["C"])
+
+
+def test_receivers_outside_the_grid_record_zero(W):
+    prob = make_problem((66, 140), 4, "dirichlet", nt=30, nrec=20, seed=9)
+    m = gpu_model(W, prob)
+    s = gpu_shots(W, prob)[0]
+    far = torch.tensor([66 * 140, 10 ** 12, -1], dtype=torch.int64, device="cuda")
+    with_far = W.Shot(s.src, s.wavelet, torch.cat([far[:1], s.rec, far[1:]]))
+    ref = m.forward([W.Shot(s.src, s.wavelet, s.rec)])[0]
+    got = m.forward([with_far])[0]
+    torch.cuda.synchronize()
+    assert torch.equal(got[1:-2], ref)
+    assert not got[0].any() and not got[-2:].any()
