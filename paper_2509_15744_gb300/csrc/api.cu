@@ -486,7 +486,7 @@ static cudaError_t run_step(const wave_model_s* m, const StepArgs& a, cudaStream
 struct TileWs {
   bool on = false;
   Tile2DPlan plan;
-  float* u[2][2];    // [pair][u^{n-1}, u^n]
+  float* u[2][2][2];   // [field][pair][u^{n-1}, u^n]
   int *count, *ptr, *cursor;
   void* ent;
   int64_t entries = 0;
@@ -502,14 +502,15 @@ struct TileWs {
 // regions (the halo work runs on SMs that would idle), a large one shallow ones.
 // Grids below 128 cells in x or 16 in y, above 2^29 cells (the second pair of
 // levels costs 2 grids) and the other storage types keep one step per launch.
-static bool tile2d_plan(const wave_model_s* m, int32_t maxrec, Tile2DPlan* out, int64_t* entries) {
+static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, Tile2DPlan* out, int64_t* entries) {
   const Geom& g = m->g;
-  if (m->d.ndim != 2 || m->d.physics != WAVE_VELOCITY || m->d.storage != WAVE_F32) return false;
+  if (m->d.ndim != 2 || m->d.storage != WAVE_F32) return false;
+  const bool tmem = m->d.physics == WAVE_DENSITY || nfields == 2;   // the tensor-memory kernel has 4 rows per warp
   if (g.nx < kStrip || g.ny < 16 || g.cells > ((int64_t)1 << 29)) return false;
   const int nx = (int)g.nx, ny = (int)g.ny, r = g.r;
   double best = 0.0;
   bool found = false;
-  for (int rb = 2; rb <= 4; rb += 2) {
+  for (int rb = tmem ? 4 : 2; rb <= 4; rb += 2) {
     const int rh = std::min(rb * 16, ny / rb * rb);
     const double step_us = std::max(0.5, rb * (0.13 + 0.04 * r));
     for (int h = 4; h <= 56; h += 4) {   // multiples of 4: owned ranges keep whole quads
@@ -544,14 +545,16 @@ static bool tile2d_plan(const wave_model_s* m, int32_t maxrec, Tile2DPlan* out, 
   return *entries < ((int64_t)1 << 30);
 }
 
-static void carve_tile(Carve& c, const wave_model_s* m, int32_t maxrec, void* u0, void* u1, TileWs* t) {
-  t->on = tile2d_plan(m, maxrec, &t->plan, &t->entries);
+// u: the first pair of levels of each field, carved by the caller.
+static void carve_tile(Carve& c, const wave_model_s* m, int32_t maxrec, int nfields, void* const* u, TileWs* t) {
+  t->on = tile2d_plan(m, nfields, maxrec, &t->plan, &t->entries);
   if (!t->on) return;
   const size_t n = (size_t)t->plan.nkx * t->plan.nky;
-  t->u[0][0] = static_cast<float*>(u0);
-  t->u[0][1] = static_cast<float*>(u1);
-  t->u[1][0] = c.take<float>(m->g.cells);
-  t->u[1][1] = c.take<float>(m->g.cells);
+  for (int f = 0; f < nfields; ++f)
+    for (int l = 0; l < 2; ++l) {
+      t->u[f][0][l] = static_cast<float*>(u[2 * f + l]);
+      t->u[f][1][l] = c.take<float>(m->g.cells);
+    }
   t->count = c.take<int>(n);
   t->cursor = c.take<int>(n);
   t->ptr = c.take<int>(n + 1);
@@ -561,9 +564,14 @@ static void carve_tile(Carve& c, const wave_model_s* m, int32_t maxrec, void* u0
 static Tile2DArgs tile_args(const wave_model_s* m, const TileWs& t, const wave_shot& sh) {
   Tile2DArgs a;
   memset(&a, 0, sizeof(a));
+  const StepArgs sa = step_args(m, nullptr, nullptr);
   a.g = m->g;
   a.plan = t.plan;
+  a.nfields = 1;
   a.coef = m->coef;
+  a.bmat = m->bmat;
+  a.da = sa.da;
+  a.dbs = sa.dbs;
   a.h2 = (float)(m->d.h * m->d.h);
   a.nrec = sh.nrec;
   a.tptr = t.ptr;
@@ -574,7 +582,8 @@ static Tile2DArgs tile_args(const wave_model_s* m, const TileWs& t, const wave_s
   return a;
 }
 
-// One launch of a.nsteps steps; the timing and metrics count every step.
+// One launch of a.nsteps steps; the timing and metrics count every step of
+// every field, as if each had been a launch.
 static cudaError_t run_tile(const wave_model_s* m, const Tile2DArgs& a, cudaStream_t s) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (g_timing.on) {
@@ -590,61 +599,71 @@ static cudaError_t run_tile(const wave_model_s* m, const Tile2DArgs& a, cudaStre
     cudaError_t err = record_event(e0, s);
     if (err != cudaSuccess) return err;
   }
-  cudaError_t err = launch_tile2d_velocity(a, m->d.order, s);
+  cudaError_t err = launch_tile2d(a, m->d.physics, m->d.order, s);
   if (err != cudaSuccess) return err;
+  const int acc_fields = !a.acc ? 0 : (a.mix ? 1 : a.nfields);
+  const int acc_steps = std::max(0, std::min(a.nsteps, a.mass_hi) - a.mass_lo);
   const double cells = (double)(m->g.nx * m->g.ny * m->g.nz);
-  const int acc_steps = a.acc ? std::max(0, std::min(a.nsteps, a.mass_hi) - a.mass_lo) : 0;
-  const double bytes = cells * (16.0 * a.nsteps + (a.comp ? 16.0 : 8.0) * acc_steps);
+  const double bytes = cells * ((m->d.physics == WAVE_DENSITY ? 20.0 : 16.0) * a.nsteps * a.nfields +
+                                (a.comp ? 16.0 : 8.0) * acc_steps * acc_fields);
   if (g_timing.on) {
     err = record_event(e1, s);
     g_timing.bytes += bytes;
-    g_timing.launches += a.nsteps;
+    g_timing.launches += a.nsteps * a.nfields;
   }
   if (m->met.on) {
     m->met.bytes += bytes;
-    m->met.launches += a.nsteps;
+    m->met.launches += a.nsteps * a.nfields;
   }
   return err;
 }
 
-// Levels u^1.. of a shot forward to u^{N+1} from pair `at` (u^0, u^1);
+// Levels u^1.. of a shot forward to u^{N+1} from pair *at (u^0, u^1);
 // records levels 1..N into what `a` names.  acc != null: -K(u,u) increments of
-// steps 1..N-1.  Returns the pair that holds (u^N, u^{N+1}) in *at.
+// steps 1..N-1.  *at becomes the pair that holds (u^N, u^{N+1}).
 static cudaError_t tile_forward(const wave_model_s* m, const TileWs& t, Tile2DArgs a, int N, int* at, cudaStream_t s) {
   a.acc_scale = 1.f;
   a.dlevel = 1;
   for (int n = 1; n <= N; n += t.plan.steps) {
     a.nsteps = std::min(t.plan.steps, N - n + 1);
     a.level0 = n;
-    a.mass_hi = N - n;
-    a.prev = t.u[*at][0];
-    a.cur = t.u[*at][1];
+    a.mass_hi = a.stiff_hi = N - n;
+    a.prev[0] = t.u[0][*at][0];
+    a.cur[0] = t.u[0][*at][1];
     *at ^= 1;
-    a.oprev = t.u[*at][0];
-    a.ocur = t.u[*at][1];
+    a.oprev[0] = t.u[0][*at][0];
+    a.ocur[0] = t.u[0][*at][1];
     cudaError_t e = run_tile(m, a, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-// The superposed pass j = N..1 from pair `at` holding (u^N, u^{N+1}).
-static cudaError_t tile_superposed(const wave_model_s* m, const TileWs& t, Tile2DArgs a, int N, int at, cudaStream_t s) {
+// The backward pass j = N..1 of a.nfields fields from pair `at` holding
+// (u^N, u^{N+1}) of each.
+static cudaError_t tile_backward(const wave_model_s* m, const TileWs& t, Tile2DArgs a, int N, int at, cudaStream_t s) {
   a.acc_scale = -1.f;
   a.dlevel = -1;
-  a.prev = t.u[at][1];
-  a.cur = t.u[at][0];
+  for (int f = 0; f < a.nfields; ++f) {
+    a.prev[f] = t.u[f][at][1];
+    a.cur[f] = t.u[f][at][0];
+  }
   for (int j = N; j >= 1; j -= t.plan.steps) {
     a.nsteps = std::min(t.plan.steps, j);
     a.level0 = j;
-    a.mass_hi = a.nsteps;
+    a.mass_hi = a.stiff_hi = a.nsteps;
+    a.stiff_lo = j == N ? 1 : 0;   // the level N is shared by u and u^s
     at ^= 1;
-    a.oprev = t.u[at][0];
-    a.ocur = t.u[at][1];
+    for (int f = 0; f < a.nfields; ++f) {
+      a.oprev[f] = t.u[f][at][0];
+      a.ocur[f] = t.u[f][at][1];
+    }
     cudaError_t e = run_tile(m, a, s);
     if (e != cudaSuccess) return e;
-    a.prev = a.oprev;
-    a.cur = a.ocur;
+    for (int f = 0; f < a.nfields; ++f) {
+      a.prev[f] = a.oprev[f];
+      a.cur[f] = a.ocur[f];
+    }
   }
   return cudaSuccess;
 }
@@ -786,7 +805,8 @@ static void carve_forward(Carve& c, const wave_model_s* m, const wave_shot* shot
   *u0 = c.take_bytes(m->g.cells * eb);
   *u1 = c.take_bytes(m->g.cells * eb);
   *recp = c.take<int64_t>(maxrec);
-  carve_tile(c, m, maxrec, *u0, *u1, tw);
+  void* const u[2] = {*u0, *u1};
+  carve_tile(c, m, maxrec, 1, u, tw);
 }
 
 extern "C" wave_status wave_forward_workspace_size(wave_model m, const wave_shot* shots, int32_t nshots,
@@ -847,8 +867,8 @@ extern "C" wave_status wave_forward(wave_model m, const wave_shot* shots, int32_
       int at = 0;
       CUDA_TRY(tile_forward(m, tw, a, N, &at, s));
       if (final_dev && si == nshots - 1) {
-        CUDA_TRY(launch_pitched_to_dense(g, tw.u[at][0], final_dev, stor, s));
-        CUDA_TRY(launch_pitched_to_dense(g, tw.u[at][1], final_dev + ncells, stor, s));
+        CUDA_TRY(launch_pitched_to_dense(g, tw.u[0][at][0], final_dev, stor, s));
+        CUDA_TRY(launch_pitched_to_dense(g, tw.u[0][at][1], final_dev + ncells, stor, s));
       }
       continue;
     }
@@ -918,7 +938,8 @@ static void carve_gradient(Carve& c, const wave_model_s* m, const wave_shot* sho
   w->recp = c.take<int64_t>(maxrec);
   w->parts = c.take<double>(1024);
   w->scal = c.take<double>(8);
-  if (!two) carve_tile(c, m, maxrec, w->u0, w->u1, &w->tile);
+  void* const u[4] = {w->u0, w->u1, w->u2, w->u3};
+  carve_tile(c, m, maxrec, two ? 2 : 1, u, &w->tile);
 }
 
 static wave_status validate_opts(const wave_model_s* m, const wave_gradient_opts* o) {
@@ -1383,8 +1404,8 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
     Tile2DArgs ta;
     if (tile) {
       ta = tile_args(m, w.tile, sh);
-      ta.acc = w.acc;
-      ta.comp = w.comp;
+      ta.acc = sym || rev ? nullptr : w.acc;   // the two-field modes need no K(u,u)
+      ta.comp = sym || rev ? nullptr : w.comp;
       CUDA_TRY(launch_tile2d_lists(w.tile.plan, g, w.recp, sh.nrec, w.tile.count, w.tile.ptr, w.tile.cursor,
                                    w.tile.ent, s));
       CUDA_TRY(launch_tile2d_skipped(w.recp, sh.nrec, 1, N, w.resid, nullptr, 0, s));
@@ -1444,6 +1465,28 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
       CUDA_TRY(launch_auto_k(w.scal + 1, w.scal + 2, ratio, wgt, kd, s));
     }
     CUDA_TRY(mark(m, kEvForwardEnd, s));
+    if (tile) {
+      // as the loops below, several steps per launch
+      float* const (&v)[2] = w.tile.u[1][at];
+      if (sym || rev) {
+        ta.nfields = 2;
+        for (int l = 0; l < 2; ++l) {
+          if (rev) CUDA_TRY(cudaMemsetAsync(v[l], 0, g.cells * eb, s));
+          else CUDA_TRY(cudaMemcpyAsync(v[l], w.tile.u[0][at][l], g.cells * eb, cudaMemcpyDeviceToDevice, s));
+        }
+      }
+      ta.mix = rev;
+      ta.src_fields = rev ? 1 : 3;
+      ta.rec_fields = rev ? 2 : 3;
+      ta.acc = w.acc;
+      ta.comp = rev ? nullptr : w.comp;
+      ta.resid_in = w.resid;
+      ta.k_dev = kd;
+      ta.weight[0] = (float)wgt;
+      ta.weight[1] = (float)(rev ? wgt : -wgt);
+      CUDA_TRY(tile_backward(m, w.tile, ta, N, at, s));
+      continue;
+    }
     // prev holds u^N, cur holds u^{N+1}
     if (rev) {
       // ---- u backward by time reversal beside lambda (Eq. kernel1 mixed term)
@@ -1555,13 +1598,6 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
         }
         for (int f = 0; f < 2; ++f) std::swap(fc[f], fn[f]);
       }
-      continue;
-    }
-    if (tile) {
-      ta.resid_in = w.resid;
-      ta.k_dev = kd;
-      ta.weight = (float)wgt;
-      CUDA_TRY(tile_superposed(m, w.tile, ta, N, at, s));
       continue;
     }
     // ---- superposed pass: u^s from (u^{N+1}, u^N), +K(u^s,u^s) ----------

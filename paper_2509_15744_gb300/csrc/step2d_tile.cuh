@@ -31,16 +31,21 @@ __host__ __device__ __forceinline__ int tile_own_hi(int k, int nk, int out, int 
 struct Tile2DArgs {
   Geom g;
   Tile2DPlan plan;
-  const float* prev;      // level n-1
-  const float* cur;       // level n
-  float* oprev;           // level n+nsteps-1 (other buffers than prev, cur)
-  float* ocur;            // level n+nsteps
+  int nfields;            // 1, or 2 that advance together
+  int mix;                // two fields u, lambda: acc -= (lambda - lambda_new)(u - u_new)
+  const float* prev[2];   // level n-1 of each field
+  const float* cur[2];    // level n
+  float* oprev[2];        // level n+nsteps-1 (other buffers than prev, cur)
+  float* ocur[2];         // level n+nsteps
   const float* coef;
+  const float* bmat;      // density form: b = 1/rho
+  float da, dbs;          // density form: as StepArgs
   float* acc;             // sensitivity accumulator (nullable), updated in place
   float* comp;            // Kahan compensation (nullable)
-  float acc_scale;        // +1 or -1
+  float acc_scale;        // +1 or -1 (one field; two have -1 and +1)
   int nsteps;             // <= plan.steps
-  int mass_lo, mass_hi;   // steps of the launch that accumulate
+  int mass_lo, mass_hi;   // steps of the launch that accumulate the (mass) term
+  int stiff_lo, stiff_hi; // density form: steps that accumulate the stiffness term
   int level0, dlevel;     // recorded / injected level of the first step, and its change per step
   // receivers (lists per region: entries ptr[t] .. ptr[t+1])
   int nrec;
@@ -53,15 +58,15 @@ struct Tile2DArgs {
   int64_t tr_ld;
   const float* resid_in;  // inject -k w e, time-major residuals (nullable)
   const double* k_dev;
-  float weight;
+  float weight[2];        // w of each field
+  int rec_fields, src_fields;   // two fields: bit f set if field f takes the receivers' / the source's force
   // source
   int sx, sy;
   const float* wavelet;   // nullable
   float h2;
 };
 
-int tile2d_smem(const Tile2DPlan& p);
-cudaError_t launch_tile2d_velocity(const Tile2DArgs& a, int order, cudaStream_t s);
+cudaError_t launch_tile2d(const Tile2DArgs& a, int physics, int order, cudaStream_t s);
 cudaError_t launch_tile2d_lists(const Tile2DPlan& p, const Geom& g, const int64_t* rec_p, int nrec, int* count,
                                 int* ptr, int* cursor, void* ent, cudaStream_t s);
 cudaError_t launch_tile2d_skipped(const int64_t* rec_p, int nrec, int lo, int hi, float* resid, float* traces,

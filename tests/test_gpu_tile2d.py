@@ -31,12 +31,18 @@ def W():
 
 
 @pytest.mark.parametrize("shape", SHAPES)
-@pytest.mark.parametrize("order,bc,nt", [(2, "dirichlet", 61), (4, "neumann", 33), (6, "dirichlet", 23),
-                                         (8, "neumann", 19), (8, "dirichlet", 1)])
-def test_forward_has_the_bits_of_single_steps(W, shape, order, bc, nt):
+@pytest.mark.parametrize("physics,order,bc,nt", [
+    ("velocity", 2, "dirichlet", 61), ("velocity", 4, "neumann", 33), ("velocity", 6, "dirichlet", 23),
+    ("velocity", 8, "neumann", 19), ("velocity", 8, "dirichlet", 1), ("density", 2, "dirichlet", 41),
+    ("density", 2, "neumann", 40)])
+def test_forward_has_the_bits_of_single_steps(W, shape, physics, order, bc, nt):
     rng = np.random.default_rng(7)
-    v = torch.from_numpy(rng.uniform(1500, 3000, shape).astype(np.float32)).cuda()
-    m = W.Model(v, 10.0, O.cfl_dt(10.0, 3000.0, 2, order, 0.5), order, "velocity", bc)
+    if physics == "velocity":
+        p, h, vmax = rng.uniform(1500, 3000, shape), 10.0, 3000.0
+    else:
+        p, h, vmax = rng.uniform(0.1, 1.0, shape), 2e-3, 509.8366
+    p = torch.from_numpy(p.astype(np.float32)).cuda()
+    m = W.Model(p, h, O.cfl_dt(h, vmax, 2, order, 0.5), order, physics, bc)
     init = torch.from_numpy(rng.standard_normal((2,) + shape).astype(np.float32)).cuda()
     none = torch.zeros(0, dtype=torch.int64, device="cuda")
     shot = W.Shot(0, torch.zeros(nt + 1, device="cuda"), none)
@@ -69,6 +75,30 @@ def test_gradient_matches_the_oracle(W, shape, order, bc, kahan, objective):
     ref = O.superposition_gradient(prob.medium(), prob.oracle_shots(), prob.nt[0], float(k.item()))
     assert rel_l2(g.cpu().numpy(), ref["K_tilde"]) < 1e-3
     assert abs(float(c.item()) - ref["C"]) < 1e-5 * abs(ref["C"])
+
+
+@pytest.mark.parametrize("shape,physics,order,bc,mode,kahan", [
+    ((65, 131), "velocity", 2, "neumann", "symmetric", False),
+    ((70, 257), "velocity", 8, "dirichlet", "symmetric", True),
+    ((66, 129), "velocity", 4, "neumann", "reverse", False),
+    ((20, 300), "velocity", 6, "dirichlet", "reverse", True)])
+def test_two_field_modes_match_the_exact_gradient(W, shape, physics, order, bc, mode, kahan):
+    prob = make_problem(shape, order, bc, physics, nt=50, nrec=60, seed=6, nshots=2)
+    m = gpu_model(W, prob, kahan=kahan)
+    g, c, _ = m.gradient(gpu_shots(W, prob), mode=mode)
+    cref, ref, _ = O.exact_gradient(prob.medium(), prob.oracle_shots(), prob.nt[0])
+    assert rel_l2(g.cpu().numpy(), ref) < 1e-3
+    assert abs(float(c.item()) - cref) < 1e-5 * abs(cref)
+
+
+def test_density_symmetric_mode_over_several_regions(W):
+    # the problem of the one-region test of this mode, on a taller grid
+    prob = make_problem((130, 150), physics="density", bc="dirichlet", nt=200, nrec=40, seed=62)
+    m = gpu_model(W, prob, kahan=True)
+    g, c, _ = m.gradient(gpu_shots(W, prob), mode="symmetric")
+    cref, ref, _ = O.exact_gradient(prob.medium(), prob.oracle_shots(), prob.nt[0])
+    assert rel_l2(g.cpu().numpy(), ref) < 1e-3
+    assert abs(float(c.item()) - cref) < 1e-5 * abs(cref)
 
 
 def test_receivers_outside_the_grid_record_zero(W):
