@@ -172,7 +172,7 @@ static Geom make_geom(const wave_grid_desc* d) {
   return g;
 }
 
-static int64_t default_zblock(const Geom& g, bool kahan) {
+static int64_t default_zblock(const Geom& g, bool kahan, bool staged) {
   const int64_t nstrips = (g.nx + kStrip - 1) / kStrip;
   if (g.ndim == 2) {
     // about 24 warps per SM over 152 SMs
@@ -181,7 +181,22 @@ static int64_t default_zblock(const Geom& g, bool kahan) {
   }
   // the largest z-block whose accumulator tile (and compensation) fits the
   // tensor memory of the batched two-shots-per-pass kernel
-  return std::min<int64_t>(kahan ? 16 : 32, g.nz);
+  const int64_t cap = std::min<int64_t>(kahan ? 16 : 32, g.nz);
+  if (!staged) return cap;
+  // The staged FP32 kernels run one CTA of 16 rows per SM, which marches its
+  // planes one after another behind a prologue worth r + 5 planes.  On a small
+  // grid deep z-blocks leave SMs idle (64 x 96 x 130: 24 CTAs at 32 planes, 49
+  // us a step; 132 at 6, 15 us), so take the depth with the least
+  // waves x (planes + prologue) over 152 SMs; the cap unless 5% better.
+  const int64_t tiles = nstrips * ((g.ny + 15) / 16);
+  auto cost = [&](int64_t zb) {
+    const int64_t waves = (tiles * ((g.nz + zb - 1) / zb) + 151) / 152;
+    return (double)waves * (double)(zb + g.r + 5);
+  };
+  int64_t best = cap;
+  for (int64_t zb = cap - 1; zb >= 2; --zb)
+    if (cost(zb) < 0.95 * cost(cap) && cost(zb) < cost(best)) best = zb;
+  return best;
 }
 
 extern "C" {
@@ -281,7 +296,7 @@ wave_status wave_model_create(const wave_grid_desc* desc, const float* param_dev
   m->param = param_dev;
   m->coef = coef;
   m->bmat = bmat;
-  m->zblock = default_zblock(g, desc->kahan != 0);
+  m->zblock = default_zblock(g, desc->kahan != 0, desc->physics == WAVE_VELOCITY && desc->storage == WAVE_F32);
   // untuned default: one field per launch on the register-queue kernel, two
   // or more on the two-shots-per-pass kernel (the faster of the batched ones
   // on every measured workload)
