@@ -172,7 +172,8 @@ static Geom make_geom(const wave_grid_desc* d) {
   return g;
 }
 
-static int64_t default_zblock(const Geom& g, bool kahan, bool staged) {
+static int64_t default_zblock(const Geom& g, const wave_grid_desc* d) {
+  const bool kahan = d->kahan != 0;
   const int64_t nstrips = (g.nx + kStrip - 1) / kStrip;
   if (g.ndim == 2) {
     // about 24 warps per SM over 152 SMs
@@ -182,7 +183,10 @@ static int64_t default_zblock(const Geom& g, bool kahan, bool staged) {
   // the largest z-block whose accumulator tile (and compensation) fits the
   // tensor memory of the batched two-shots-per-pass kernel
   const int64_t cap = std::min<int64_t>(kahan ? 16 : 32, g.nz);
-  if (!staged) return cap;
+  if (d->storage != WAVE_F32) return cap;
+  // density: warps march without staging; 8 planes give enough of them (180 x
+  // 210 x 250: 73 us per field and step at 8, 81 at 10, 87 at 15, 82 at 20)
+  if (d->physics == WAVE_DENSITY) return std::min<int64_t>(8, g.nz);
   // The staged FP32 kernels run one CTA of 16 rows per SM, which marches its
   // planes one after another behind a prologue worth r + 5 planes.  On a small
   // grid deep z-blocks leave SMs idle (64 x 96 x 130: 24 CTAs at 32 planes, 49
@@ -296,7 +300,7 @@ wave_status wave_model_create(const wave_grid_desc* desc, const float* param_dev
   m->param = param_dev;
   m->coef = coef;
   m->bmat = bmat;
-  m->zblock = default_zblock(g, desc->kahan != 0, desc->physics == WAVE_VELOCITY && desc->storage == WAVE_F32);
+  m->zblock = default_zblock(g, desc);
   // untuned default: one field per launch on the register-queue kernel, two
   // or more on the two-shots-per-pass kernel (the faster of the batched ones
   // on every measured workload)
@@ -461,6 +465,7 @@ static double step_bytes(const wave_model_s* m, const StepArgs& a) {
   double b = 3.0 * eb + 4.0;                    // read u^n, u^{n-1}, coef; write u^{n+1}
   if (m->d.physics == WAVE_DENSITY) b += 4.0;   // read b
   if (a.acc_mass || a.acc_stiff) b += a.comp ? 16.0 : 8.0;  // accumulator (+ compensation) RMW
+  if (a.u_cur2) b *= 2.0;                       // counted per field, as two launches
   return cells * b;
 }
 
@@ -485,11 +490,11 @@ static cudaError_t run_step(const wave_model_s* m, const StepArgs& a, cudaStream
   if (g_timing.on) {
     err = record_event(e1, s);
     g_timing.bytes += step_bytes(m, a);
-    g_timing.launches += 1;
+    g_timing.launches += a.u_cur2 ? 2 : 1;
   }
   if (m->met.on) {
     m->met.bytes += step_bytes(m, a);
-    m->met.launches += 1;
+    m->met.launches += a.u_cur2 ? 2 : 1;
   }
   return err;
 }
@@ -1396,6 +1401,7 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
   const double ratio = default_ratio(m, opts);
   // both fields of WAVE_SYMMETRIC_K advance in one launch where the batched kernel applies
   const bool fuse2 = sym && m->d.ndim == 3 && m->d.physics == WAVE_VELOCITY && stor == WAVE_F32;
+  const bool den2 = sym && m->d.ndim == 3 && m->d.physics == WAVE_DENSITY && stor == WAVE_F32;
 
   for (int si = 0; si < nshots; ++si) {
     const wave_shot& sh = shots[si];
@@ -1600,6 +1606,17 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
             b.accf[f] = f == 0 ? 1.f : -1.f;   // -K(u^+,u^+) ... +K(u^-,u^-)
           }
           CUDA_TRY(run_batched(m, b, s));
+        } else if (den2) {
+          StepArgs a = step_args(m, fc[0], fn[0]);
+          a.u_cur2 = fc[1];
+          a.u_prev2 = fn[1];
+          a.acc = w.acc;
+          a.comp = w.comp;
+          a.acc_scale = -1.f;
+          a.acc_scale2 = 1.f;
+          a.acc_mass = 1;
+          a.acc_stiff = j <= N - 1;
+          CUDA_TRY(run_step(m, a, s));
         } else {
           for (int f = 0; f < 2; ++f) {
             StepArgs a = step_args(m, fc[f], fn[f]);

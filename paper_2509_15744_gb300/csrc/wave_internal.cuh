@@ -143,6 +143,10 @@ struct StepArgs {
   // Exact (stored-history) mode, FP32 velocity only:
   const float* mix_a;    // stored u^j (nullable): accumulate the mixed term
   const float* mix_b;    // stored u^{j-1}: acc += acc_scale (u_cur - u_next)(mix_a - mix_b)
+  // 3D density form, FP32: a second field advanced in the same launch (nullable)
+  const void* u_cur2;
+  void* u_prev2;
+  float acc_scale2;
 };
 
 // Launchers (defined in step_*.cu).  Return cudaGetLastError() of the launch.
