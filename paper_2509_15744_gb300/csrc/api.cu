@@ -513,13 +513,16 @@ struct TileWs {
 };
 
 // Region split for the model's 2D grid: rows per warp (2 or 4; 16 warps) and
-// steps per launch S that minimise the modelled time of a step,
-//   (launch + waves * (edge + S * step)) / S,
-// over 152 CTAs a wave.  The figures are fits to measured gradient calls (128^2
-// and 251^2 order 2, 2048^2 order 8, 6001 x 8003 order 4 on GB300): about 5 us
-// for a region's loads, lists and stores, 1 us a launch, and per step
-// rb (0.13 + 0.04 r) us but at least 0.5.  A small grid thus takes deep
-// regions (the halo work runs on SMs that would idle), a large one shallow ones.
+// steps per launch S with the least modelled time of a step.  The figures are
+// fits to measured gradient calls on GB300 (128^2, 251^2, 363^2, 2048^2, 6001 x
+// 8003, orders 2-8), us:
+//   all regions at once (152 SMs), launches overlapping:
+//     (2.6 + S (0.34 + 0.22 r)) / S with 2 rows, (3.4 + S (0.5 + 0.38 r)) / S with 4;
+//   several waves: (1 + waves (5 + S rb (0.13 + 0.04 r))) / S.
+// A small grid thus takes deep regions (the halo work runs on SMs that would
+// idle), a large one shallow ones.  Measured at the fits' choices and next to
+// them, 251^2 order 2, 6400 steps: 2 rows S = 12 5.1 ms (8: 5.6, 4: 7.6), 4 rows
+// S = 24 6.8; 2048^2 order 8, 800 steps: 4 rows S = 3 16.4 ms (2: 19.1).
 // Grids below 128 cells in x or 16 in y, above 2^29 cells (the second pair of
 // levels costs 2 grids) and the other storage types keep one step per launch.
 static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, Tile2DPlan* out, int64_t* entries) {
@@ -532,7 +535,6 @@ static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, Tile
   bool found = false;
   for (int rb = tmem ? 4 : 2; rb <= 4; rb += 2) {
     const int rh = std::min(rb * 16, ny / rb * rb);
-    const double step_us = std::max(0.5, rb * (0.13 + 0.04 * r));
     for (int h = 4; h <= 56; h += 4) {   // multiples of 4: owned ranges keep whole quads
       if (h % r) continue;
       Tile2DPlan p;
@@ -548,8 +550,10 @@ static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, Tile
       if (p.nkx == 1) p.outx = kStrip;
       if (p.nky == 1) p.outy = rh;
       if (p.nky > 65535) continue;
-      const double waves = ceil((double)p.nkx * p.nky / 152.0);
-      const double t = (1.0 + waves * (5.0 + p.steps * step_us)) / p.steps;
+      const double waves = ceil((double)p.nkx * p.nky / 152.0), S = p.steps;
+      const double t = waves > 1.0 ? (1.0 + waves * (5.0 + S * rb * (0.13 + 0.04 * r))) / S
+                       : rb == 2   ? (2.6 + S * (0.34 + 0.22 * r)) / S
+                                   : (3.4 + S * (0.5 + 0.38 * r)) / S;
       if (!found || t < best) {
         best = t;
         *out = p;
@@ -638,6 +642,13 @@ static cudaError_t run_tile(const wave_model_s* m, const Tile2DArgs& a, cudaStre
   return err;
 }
 
+// Launches of one pass overlap (the next one's lists and coefficients load
+// while the last one ends) where a launch leaves SMs free for it; not while
+// events are recorded between them.
+static bool tile_overlap(const wave_model_s* m, const TileWs& t) {
+  return t.plan.nkx * t.plan.nky <= 152 && !g_timing.on && !m->met.on;
+}
+
 // Levels u^1.. of a shot forward to u^{N+1} from pair *at (u^0, u^1);
 // records levels 1..N into what `a` names.  acc != null: -K(u,u) increments of
 // steps 1..N-1.  *at becomes the pair that holds (u^N, u^{N+1}).
@@ -646,6 +657,7 @@ static cudaError_t tile_forward(const wave_model_s* m, const TileWs& t, Tile2DAr
   a.dlevel = 1;
   for (int n = 1; n <= N; n += t.plan.steps) {
     a.nsteps = std::min(t.plan.steps, N - n + 1);
+    a.overlap = n > 1 && tile_overlap(m, t);
     a.level0 = n;
     a.mass_hi = a.stiff_hi = N - n;
     a.prev[0] = t.u[0][*at][0];
@@ -670,6 +682,7 @@ static cudaError_t tile_backward(const wave_model_s* m, const TileWs& t, Tile2DA
   }
   for (int j = N; j >= 1; j -= t.plan.steps) {
     a.nsteps = std::min(t.plan.steps, j);
+    a.overlap = j < N && tile_overlap(m, t);
     a.level0 = j;
     a.mass_hi = a.stiff_hi = a.nsteps;
     a.stiff_lo = j == N ? 1 : 0;   // the level N is shared by u and u^s

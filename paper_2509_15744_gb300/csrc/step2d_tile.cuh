@@ -44,6 +44,7 @@ struct Tile2DArgs {
   float* comp;            // Kahan compensation (nullable)
   float acc_scale;        // +1 or -1 (one field; two have -1 and +1)
   int nsteps;             // <= plan.steps
+  int overlap;            // the launch before in the stream is a step of the same pass: start while it ends
   int mass_lo, mass_hi;   // steps of the launch that accumulate the (mass) term
   int stiff_lo, stiff_hi; // density form: steps that accumulate the stiffness term
   int level0, dlevel;     // recorded / injected level of the first step, and its change per step
@@ -67,6 +68,11 @@ struct Tile2DArgs {
 };
 
 cudaError_t launch_tile2d(const Tile2DArgs& a, int physics, int order, cudaStream_t s);
+cudaError_t launch_tile2d_o2(const Tile2DArgs& a, cudaStream_t s);   // one translation unit each
+cudaError_t launch_tile2d_o4(const Tile2DArgs& a, cudaStream_t s);
+cudaError_t launch_tile2d_o6(const Tile2DArgs& a, cudaStream_t s);
+cudaError_t launch_tile2d_o8(const Tile2DArgs& a, cudaStream_t s);
+cudaError_t launch_tile2d_density(const Tile2DArgs& a, cudaStream_t s);
 cudaError_t launch_tile2d_lists(const Tile2DPlan& p, const Geom& g, const int64_t* rec_p, int nrec, int* count,
                                 int* ptr, int* cursor, void* ent, cudaStream_t s);
 cudaError_t launch_tile2d_skipped(const int64_t* rec_p, int nrec, int lo, int hi, float* resid, float* traces,

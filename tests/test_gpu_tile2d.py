@@ -112,3 +112,28 @@ def test_receivers_outside_the_grid_record_zero(W):
     torch.cuda.synchronize()
     assert torch.equal(got[1:-2], ref)
     assert not got[0].any() and not got[-2:].any()
+
+
+@pytest.mark.parametrize("physics,mode", [("velocity", "superposition"), ("velocity", "reverse"),
+                                          ("density", "symmetric")])
+def test_overlapping_launches_captured_in_a_cuda_graph(W, physics, mode):
+    # the launches of a pass start while the one before ends; captured, replayed
+    # and on another stream they give the bits of the eager call
+    prob = make_problem((70, 150), 2, "neumann", physics, nt=90, nrec=30, seed=11)
+    m, shots = gpu_model(W, prob), gpu_shots(W, prob)
+    eager, c, _ = m.gradient(shots, mode=mode, k=1.0)
+    out = torch.empty_like(eager)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        _, cg, _ = m.gradient(shots, mode=mode, k=1.0, out=out)
+    for _ in range(2):
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, eager) and float(cg.item()) == float(c.item())
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        again, c2, _ = m.gradient(shots, mode=mode, k=1.0)
+    side.synchronize()
+    assert torch.equal(again, eager) and float(c2.item()) == float(c.item())
