@@ -45,51 +45,83 @@ static unsigned grid_for(int64_t n, int threads) {
   return (unsigned)b;
 }
 
+// Grid passes: a warp takes pieces of at most kPiece cells of a row, lanes along
+// x, so no cell needs a division (the 64-bit ones per cell made a layout
+// conversion of 48e6 cells take 240 us, 5x its bytes at the copy bandwidth).
+// f(row, x, index in the dense grid, index in the pitched grid) is called for
+// every x < xmax (nx, or px where the padding is written too).
+constexpr int kPiece = 1024;
+template <typename F>
+__device__ __forceinline__ void for_cells(const Geom& g, int64_t xmax, F f) {
+  const int lane = threadIdx.x & 31;
+  const int64_t rows = g.ny * g.nz;
+  const unsigned pieces = (unsigned)((xmax + kPiece - 1) / kPiece);
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  int64_t row = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) / pieces;
+  unsigned piece = (unsigned)(((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) - row * pieces);
+  const int64_t drow = nwarps / pieces;
+  const unsigned dpiece = (unsigned)(nwarps - drow * pieces);
+  while (row < rows) {
+    const int64_t x0 = (int64_t)piece * kPiece, x1 = x0 + kPiece < xmax ? x0 + kPiece : xmax;
+    const int64_t dense = row * g.nx, pitched = row * g.px;
+#pragma unroll 4
+    for (int64_t x = x0 + lane; x < x1; x += 32) f(row, x, dense + x, pitched + x);
+    row += drow;
+    piece += dpiece;
+    if (piece >= pieces) {
+      piece -= pieces;
+      ++row;
+    }
+  }
+}
+static unsigned grid_for_rows(const Geom& g, int64_t xmax, int threads) {
+  const int64_t items = g.ny * g.nz * ((xmax + kPiece - 1) / kPiece), per = threads / 32;
+  int64_t b = (items + per - 1) / per;
+  if (b > 152 * 16) b = 152 * 16;   // 16 CTAs of 8 warps fill an SM twice over
+  return (unsigned)(b < 1 ? 1 : b);
+}
+
 // ---- materials of the acoustic model (Sec. 2.3) ---------------------------
 constexpr double kRhoAir = 1.204, kKappaAir = 1.419e5;
 constexpr double kRhoSolid = 2643.0, kKappaSolid = 6.87e8;
 
 __global__ void coef_velocity_kernel(Geom g, const float* __restrict__ v, float dt_over_h,
                                      float* __restrict__ coef) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.cells;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t x = i % g.px, row = i / g.px;
+  for_cells(g, g.px, [&](int64_t, int64_t x, int64_t i, int64_t p) {
     float c = 0.f;
     if (x < g.nx) {
-      const float s = v[row * g.nx + x] * dt_over_h;
+      const float s = v[i] * dt_over_h;
       c = s * s;
     }
-    coef[i] = c;
-  }
+    coef[p] = c;
+  });
 }
 
 __global__ void coef_density_kernel(Geom g, const float* __restrict__ gamma, double dt2_over_h2,
                                     float* __restrict__ ca, float* __restrict__ b) {
   const double a_air = 1.0 / kKappaAir, da = 1.0 / kKappaSolid - 1.0 / kKappaAir;
   const double b_air = 1.0 / kRhoAir, db = 1.0 / kRhoSolid - 1.0 / kRhoAir;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.cells;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t x = i % g.px, row = i / g.px;
+  for_cells(g, g.px, [&](int64_t, int64_t x, int64_t i, int64_t p) {
     float cav = 0.f, bv = 1.f;  // padding: no mass term, unit (finite) material
     if (x < g.nx) {
-      const double gm = gamma[row * g.nx + x];
+      const double gm = gamma[i];
       cav = (float)(dt2_over_h2 / (a_air + gm * da));
       bv = (float)(b_air + gm * db);
     }
-    ca[i] = cav;
-    b[i] = bv;
-  }
+    ca[p] = cav;
+    b[p] = bv;
+  });
 }
 
 cudaError_t launch_coef_velocity(const Geom& g, const float* v, float dt_over_h, float* coef, cudaStream_t s) {
-  coef_velocity_kernel<<<grid_for(g.cells, 256), 256, 0, s>>>(g, v, dt_over_h, coef);
+  coef_velocity_kernel<<<grid_for_rows(g, g.px, 256), 256, 0, s>>>(g, v, dt_over_h, coef);
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_coef_density(const Geom& g, const float* gamma, double dt2_over_h2, float* ca, float* b,
                                 cudaStream_t s) {
-  coef_density_kernel<<<grid_for(g.cells, 256), 256, 0, s>>>(g, gamma, dt2_over_h2, ca, b);
+  coef_density_kernel<<<grid_for_rows(g, g.px, 256), 256, 0, s>>>(g, gamma, dt2_over_h2, ca, b);
   count_launch();
   return cudaGetLastError();
 }
@@ -109,15 +141,17 @@ __global__ void stability_kernel(Geom g, int physics, float sym, const float* __
                                  const float* __restrict__ b, float* __restrict__ partial) {
   __shared__ float red[256];
   float m = 0.f;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.cells;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t x = i % g.px;
-    if (x >= g.nx) continue;
+  int64_t last = -1, y = 0, z = 0;   // row of the cell before, and its place
+  for_cells(g, g.nx, [&](int64_t row, int64_t x, int64_t, int64_t i) {
     float val;
     if (physics == WAVE_VELOCITY) {
       val = coef[i] * sym;
     } else {
-      const int64_t row = i / g.px, y = row % g.ny, z = row / g.ny;
+      if (row != last) {
+        last = row;
+        z = row / g.ny;
+        y = row - z * g.ny;
+      }
       const float bi = b[i];
       float s = 0.f;
       const float edge = g.bc == WAVE_DIRICHLET ? bi : 0.f;
@@ -132,7 +166,7 @@ __global__ void stability_kernel(Geom g, int physics, float sym, const float* __
       val = 2.f * coef[i] * s;
     }
     m = max_keep_nan(m, val);
-  }
+  });
   red[threadIdx.x] = m;
   __syncthreads();
   for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -187,24 +221,16 @@ cudaError_t launch_pitch_indices(const Geom& g, const int64_t* flat, int32_t n, 
 
 template <typename T>
 __global__ void dense_to_pitched_kernel(Geom g, const float* __restrict__ dense, T* __restrict__ out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.cells;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t x = i % g.px, row = i / g.px;
-    out[i] = T(x < g.nx ? dense[row * g.nx + x] : 0.f);
-  }
+  for_cells(g, g.px, [&](int64_t, int64_t x, int64_t i, int64_t p) { out[p] = T(x < g.nx ? dense[i] : 0.f); });
 }
 
 template <typename T>
 __global__ void pitched_to_dense_kernel(Geom g, const T* __restrict__ in, float* __restrict__ dense) {
-  const int64_t total = g.nx * g.ny * g.nz;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    dense[i] = float(in[(i / g.nx) * g.px + (i % g.nx)]);
-  }
+  for_cells(g, g.nx, [&](int64_t, int64_t, int64_t i, int64_t p) { dense[i] = float(in[p]); });
 }
 
 cudaError_t launch_dense_to_pitched(const Geom& g, const float* dense, void* pitched, int storage, cudaStream_t s) {
-  const unsigned grid = grid_for(g.cells, 256);
+  const unsigned grid = grid_for_rows(g, g.px, 256);
   if (storage == WAVE_F32) dense_to_pitched_kernel<float><<<grid, 256, 0, s>>>(g, dense, (float*)pitched);
   else if (storage == WAVE_BF16) dense_to_pitched_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(g, dense, (__nv_bfloat16*)pitched);
   else dense_to_pitched_kernel<__half><<<grid, 256, 0, s>>>(g, dense, (__half*)pitched);
@@ -213,7 +239,7 @@ cudaError_t launch_dense_to_pitched(const Geom& g, const float* dense, void* pit
 }
 
 cudaError_t launch_pitched_to_dense(const Geom& g, const void* pitched, float* dense, int storage, cudaStream_t s) {
-  const unsigned grid = grid_for(g.nx * g.ny * g.nz, 256);
+  const unsigned grid = grid_for_rows(g, g.nx, 256);
   if (storage == WAVE_F32) pitched_to_dense_kernel<float><<<grid, 256, 0, s>>>(g, (const float*)pitched, dense);
   else if (storage == WAVE_BF16) pitched_to_dense_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(g, (const __nv_bfloat16*)pitched, dense);
   else pitched_to_dense_kernel<__half><<<grid, 256, 0, s>>>(g, (const __half*)pitched, dense);
@@ -377,18 +403,16 @@ __global__ void finish_kernel(Geom g, const float* __restrict__ acc, const doubl
   __shared__ double red[32];
   const double sc = superposition ? inv_dt / (2.0 * k_dev[0]) : inv_dt;
   const float s = (float)sc;
-  const int64_t total = g.nx * g.ny * g.nz;
   double ss = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    float v = acc[(i / g.nx) * g.px + (i % g.nx)] * s;
+  for_cells(g, g.nx, [&](int64_t, int64_t, int64_t i, int64_t q) {
+    float v = acc[q] * s;
     if (chain_v) {
       const float p = param[i];
       v *= -2.f / (p * p * p);   // dC/dv = dC/dm * dm/dv, m = 1/v^2
     }
     grad[i] = v;
     ss = fma((double)v, (double)v, ss);
-  }
+  });
   const double bs = block_sum(ss, red);
   if (threadIdx.x == 0) partial[blockIdx.x] = bs;
 }

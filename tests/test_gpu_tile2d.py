@@ -19,7 +19,7 @@ from _problems import make_problem, rel_l2
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(16, 128), (17, 129), (64, 128), (65, 131), (130, 257), (203, 383)]
+SHAPES = [(16, 128), (17, 129), (64, 128), (65, 131), (130, 257), (203, 383), (19, 2501)]
 
 
 @pytest.fixture(scope="module")
