@@ -176,9 +176,12 @@ static int64_t default_zblock(const Geom& g, const wave_grid_desc* d) {
   const bool kahan = d->kahan != 0;
   const int64_t nstrips = (g.nx + kStrip - 1) / kStrip;
   if (g.ndim == 2) {
-    // about 24 warps per SM over 152 SMs
+    // about 24 warps per SM over 152 SMs; a row's loads follow the last row's,
+    // so small grids take one row per warp (100^2, order 2: 4.6 us a step with
+    // its source / receiver launch, 11.5 at 8 rows; 1400^2 order 8: 4 and 8 rows
+    // alike, one row 1.5 times slower)
     int64_t by = nstrips * g.ny / (152 * 24);
-    return std::max<int64_t>(8, std::min<int64_t>(by, 256));
+    return std::max<int64_t>(1, std::min<int64_t>(by, 256));
   }
   // the largest z-block whose accumulator tile (and compensation) fits the
   // tensor memory of the batched two-shots-per-pass kernel
