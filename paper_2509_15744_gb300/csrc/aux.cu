@@ -258,6 +258,7 @@ cudaError_t launch_pitched_to_dense(const Geom& g, const void* pitched, float* d
 //           (receivers, Eq. superposedforce).  Atomic: cells may repeat.
 template <typename T>
 __global__ void sparse_kernel(SparseArgs a) {
+  chain_wait();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t < a.nrec) {
     const int64_t p = a.rec_p[t];
@@ -293,11 +294,10 @@ __global__ void sparse_kernel(SparseArgs a) {
 cudaError_t launch_sparse(const SparseArgs& a, int storage, cudaStream_t s) {
   const int64_t n = (int64_t)a.nrec + 1;
   const unsigned grid = (unsigned)((n + 255) / 256);
-  if (storage == WAVE_F32) sparse_kernel<float><<<grid, 256, 0, s>>>(a);
-  else if (storage == WAVE_BF16) sparse_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(a);
-  else sparse_kernel<__half><<<grid, 256, 0, s>>>(a);
   count_launch();
-  return cudaGetLastError();
+  if (storage == WAVE_F32) return launch_chained(sparse_kernel<float>, grid, 256, 0, s, a);
+  if (storage == WAVE_BF16) return launch_chained(sparse_kernel<__nv_bfloat16>, grid, 256, 0, s, a);
+  return launch_chained(sparse_kernel<__half>, grid, 256, 0, s, a);
 }
 
 // ---- FP64 reductions -----------------------------------------------------

@@ -127,6 +127,7 @@ step3d_velocity_pair_kernel(BatchArgs b) {
   constexpr int D = PT::D;
   constexpr int NB = PT::NB;
   extern __shared__ __align__(16) float tiles[];   // [2][NB][TILE]
+  chain_wait();
   const StepArgs& a = b.base;
   const Geom& g = a.g;
   const int tid = threadIdx.x;
@@ -228,8 +229,8 @@ step3d_velocity_pair_kernel(BatchArgs b) {
   for (int s0 = 0; s0 < b.nshots; s0 += 2) {
     const bool first = s0 == 0, last = s0 + 2 >= b.nshots;
     const bool two = s0 + 1 < b.nshots;   // uniform: a second field in this pass
-    const float* __restrict__ ucA = b.cur[s0];
-    const float* __restrict__ ucB = two ? b.cur[s0 + 1] : b.cur[s0];
+    const float* __restrict__ ucA = after_wait(b.cur[s0]);
+    const float* __restrict__ ucB = after_wait(two ? b.cur[s0 + 1] : b.cur[s0]);
     float* __restrict__ upA = b.prev[s0];
     float* __restrict__ upB = two ? b.prev[s0 + 1] : b.prev[s0];
     const float fA = b.accf[s0], fB = two ? b.accf[s0 + 1] : 0.f;
@@ -468,9 +469,8 @@ cudaError_t launch_p(const BatchArgs& b, cudaStream_t s) {
   const unsigned nzb = (unsigned)((g.nz + b.base.zblock - 1) / b.base.zblock);
   const unsigned nxs = (unsigned)((g.nx + kStrip - 1) / kStrip), nyt = (unsigned)((g.ny + TY - 1) / TY);
   const dim3 grid = b.base.cta_order ? dim3(nxs, nyt, nzb) : dim3(nzb, nxs, nyt);
-  step3d_velocity_pair_kernel<R, TY, DX, ACC, TM><<<grid, TY * 32, PT::bytes(), s>>>(b);
+  e = launch_chained(step3d_velocity_pair_kernel<R, TY, DX, ACC, TM>, grid, TY * 32, PT::bytes(), s, b);
   count_launch();
-  e = cudaGetLastError();
   if (e != cudaSuccess) note_error("step kernel launch", e);
   return e;
 }

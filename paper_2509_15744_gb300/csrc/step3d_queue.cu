@@ -64,6 +64,7 @@ step3d_velocity_queue_kernel(BatchArgs b) {
   constexpr int D = QT::D;
   constexpr int NB = QT::NB;
   extern __shared__ __align__(16) float tiles[];
+  chain_wait();
   const StepArgs& a = b.base;
   const Geom& g = a.g;
   const int tid = threadIdx.x;
@@ -137,7 +138,7 @@ step3d_velocity_queue_kernel(BatchArgs b) {
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
 
   for (int shot = 0; shot < b.nshots; ++shot) {
-    const float* __restrict__ uc = b.cur[shot];
+    const float* __restrict__ uc = after_wait(b.cur[shot]);
     float* __restrict__ up = b.prev[shot];
     const bool acc_on = b.accf[shot] != 0;
     const float acc_sc = a.acc_scale * b.accf[shot];  // per-shot sign and on/off
@@ -314,9 +315,8 @@ cudaError_t launch_q(const BatchArgs& b, cudaStream_t s) {
   const unsigned nzb = (unsigned)((g.nz + b.base.zblock - 1) / b.base.zblock);
   const unsigned nxs = (unsigned)((g.nx + kStrip - 1) / kStrip), nyt = (unsigned)((g.ny + TY - 1) / TY);
   const dim3 grid = b.base.cta_order ? dim3(nxs, nyt, nzb) : dim3(nzb, nxs, nyt);
-  step3d_velocity_queue_kernel<R, TY, DX><<<grid, TY * 32, QT::bytes(), s>>>(b);
+  e = launch_chained(step3d_velocity_queue_kernel<R, TY, DX>, grid, TY * 32, QT::bytes(), s, b);
   count_launch();
-  e = cudaGetLastError();
   if (e != cudaSuccess) note_error("step kernel launch", e);
   return e;
 }

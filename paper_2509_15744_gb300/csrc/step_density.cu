@@ -78,6 +78,7 @@ __device__ __forceinline__ void stage_row(float* srow, const T* __restrict__ f, 
 template <typename T, int WPB>
 __global__ void __launch_bounds__(WPB * 32)
 step2d_density_kernel(StepArgs a) {
+  chain_wait();
   __shared__ __align__(16) float su[WPB][kRowW];
   __shared__ __align__(16) float sb[WPB][kRowW];
   const Geom& g = a.g;
@@ -92,8 +93,8 @@ step2d_density_kernel(StepArgs a) {
   const int64_t x0 = strip * kStrip;
   const int64_t xl = x0 + 4 * lane;
   const bool xin = (x0 >= 4) && (x0 + kStrip + 4 <= g.nx);
-  const T* __restrict__ uc = reinterpret_cast<const T*>(a.u_cur);
-  const T* __restrict__ up = reinterpret_cast<const T*>(a.u_prev);
+  const T* __restrict__ uc = after_wait(reinterpret_cast<const T*>(a.u_cur));
+  const T* __restrict__ up = after_wait(reinterpret_cast<const T*>(a.u_prev));
   const float* __restrict__ bm = a.bmat;
   const bool dir = g.bc == WAVE_DIRICHLET;
   for (int i = lane; i < kRowW; i += 32) { su[warp][i] = 0.f; sb[warp][i] = 1.f; }
@@ -184,6 +185,7 @@ step2d_density_kernel(StepArgs a) {
 template <typename T, int WPB>
 __global__ void __launch_bounds__(WPB * 32)
 step3d_density_kernel(StepArgs a) {
+  chain_wait();
   __shared__ __align__(16) float su[WPB][kRowW];
   __shared__ __align__(16) float sb[WPB][kRowW];
   const Geom& g = a.g;
@@ -202,8 +204,8 @@ step3d_density_kernel(StepArgs a) {
   const int64_t x0 = strip * kStrip;
   const int64_t xl = x0 + 4 * lane;
   const bool xin = (x0 >= 4) && (x0 + kStrip + 4 <= g.nx);
-  const T* __restrict__ uc = reinterpret_cast<const T*>(a.u_cur);
-  const T* __restrict__ up = reinterpret_cast<const T*>(a.u_prev);
+  const T* __restrict__ uc = after_wait(reinterpret_cast<const T*>(a.u_cur));
+  const T* __restrict__ up = after_wait(reinterpret_cast<const T*>(a.u_prev));
   const float* __restrict__ bm = a.bmat;
   const bool dir = g.bc == WAVE_DIRICHLET;
   for (int i = lane; i < kRowW; i += 32) { su[warp][i] = 0.f; sb[warp][i] = 1.f; }
@@ -320,6 +322,7 @@ constexpr int kMarchRows = 8;
 template <int NF, int ACC>   // ACC: 0 none, 1 acc, 2 with compensation
 __global__ void __launch_bounds__(kMarchRows * 32, ACC == 0 ? 3 : 2)
 step3d_density_march_kernel(StepArgs a) {
+  chain_wait();
   const Geom& g = a.g;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t nstrips = (g.nx + kStrip - 1) / kStrip, nyt = (g.ny + kMarchRows - 1) / kMarchRows;
@@ -335,10 +338,10 @@ step3d_density_march_kernel(StepArgs a) {
   const float* const bm = a.bmat;
   const float* uc[NF];
   float* up[NF];
-  uc[0] = reinterpret_cast<const float*>(a.u_cur);
+  uc[0] = after_wait(reinterpret_cast<const float*>(a.u_cur));
   up[0] = reinterpret_cast<float*>(a.u_prev);
   if constexpr (NF == 2) {
-    uc[1] = reinterpret_cast<const float*>(a.u_cur2);
+    uc[1] = after_wait(reinterpret_cast<const float*>(a.u_cur2));
     up[1] = reinterpret_cast<float*>(a.u_prev2);
   }
   auto ld = [](const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); };
@@ -539,11 +542,10 @@ static cudaError_t launch_march(const StepArgs& a, cudaStream_t s) {
   const int64_t blocks = (g.nx + kStrip - 1) / kStrip * ((g.ny + kMarchRows - 1) / kMarchRows) *
                          ((g.nz + a.zblock - 1) / a.zblock);
   const bool acc = a.acc_mass || a.acc_stiff;
-  if (!acc) step3d_density_march_kernel<NF, 0><<<(unsigned)blocks, kMarchRows * 32, 0, s>>>(a);
-  else if (!a.comp) step3d_density_march_kernel<NF, 1><<<(unsigned)blocks, kMarchRows * 32, 0, s>>>(a);
-  else step3d_density_march_kernel<NF, 2><<<(unsigned)blocks, kMarchRows * 32, 0, s>>>(a);
   count_launch();
-  return cudaGetLastError();
+  if (!acc) return launch_chained(step3d_density_march_kernel<NF, 0>, (unsigned)blocks, kMarchRows * 32, 0, s, a);
+  if (!a.comp) return launch_chained(step3d_density_march_kernel<NF, 1>, (unsigned)blocks, kMarchRows * 32, 0, s, a);
+  return launch_chained(step3d_density_march_kernel<NF, 2>, (unsigned)blocks, kMarchRows * 32, 0, s, a);
 }
 
 constexpr int kWarpsDen = 4;
@@ -558,17 +560,15 @@ static cudaError_t launch_den(const StepArgs& a, cudaStream_t s) {
     } else {
       const int64_t warps = nstrips * g.ny * ((g.nz + a.zblock - 1) / a.zblock);
       const int64_t blocks = (warps + kWarpsDen - 1) / kWarpsDen;
-      step3d_density_kernel<T, kWarpsDen><<<(unsigned)blocks, kWarpsDen * 32, 0, s>>>(a);
       count_launch();
-      return cudaGetLastError();
+      return launch_chained(step3d_density_kernel<T, kWarpsDen>, (unsigned)blocks, kWarpsDen * 32, 0, s, a);
     }
   }
   if (g.ndim != 2) return cudaErrorInvalidValue;
   const int64_t warps = nstrips * ((g.ny + a.zblock - 1) / a.zblock);
   const int64_t blocks = (warps + kWarpsDen - 1) / kWarpsDen;
-  step2d_density_kernel<T, kWarpsDen><<<(unsigned)blocks, kWarpsDen * 32, 0, s>>>(a);
   count_launch();
-  return cudaGetLastError();
+  return launch_chained(step2d_density_kernel<T, kWarpsDen>, (unsigned)blocks, kWarpsDen * 32, 0, s, a);
 }
 
 cudaError_t launch_step_density(const StepArgs& a, int storage, cudaStream_t s) {

@@ -72,6 +72,7 @@ template <int R, typename T, int WPB>
 __global__ void __launch_bounds__(WPB * 32)
 step2d_velocity_kernel(StepArgs a) {
   __shared__ __align__(16) float sm[WPB][kRowW];
+  chain_wait();
   const Geom& g = a.g;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -84,8 +85,8 @@ step2d_velocity_kernel(StepArgs a) {
   const int64_t x0 = strip * kStrip;
   const int64_t xl = x0 + 4 * lane;
   const bool xin = (x0 >= 4) && (x0 + kStrip + 4 <= g.nx);
-  const T* __restrict__ uc = reinterpret_cast<const T*>(a.u_cur);
-  const T* __restrict__ up = reinterpret_cast<const T*>(a.u_prev);
+  const T* __restrict__ uc = after_wait(reinterpret_cast<const T*>(a.u_cur));
+  const T* __restrict__ up = after_wait(reinterpret_cast<const T*>(a.u_prev));
   float* srow = sm[warp];
   // Staged rows start at zero so that never-written halo slots are finite.
   for (int i = lane; i < kRowW; i += 32) srow[i] = 0.f;
@@ -137,6 +138,7 @@ __global__ void __launch_bounds__(TY * 32, R >= 3 ? 4 : 1)
 step3d_velocity_kernel(StepArgs a) {
   static_assert(TY >= 2 * R, "the first 2r warps stage the y halo rows");
   __shared__ __align__(16) float sm[2][TY + 2 * R][kRowW];
+  chain_wait();
   const Geom& g = a.g;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -147,8 +149,8 @@ step3d_velocity_kernel(StepArgs a) {
   const int64_t z1 = min(z0 + a.zblock, g.nz);
   const int64_t xl = x0 + 4 * lane;
   const bool xin = (x0 >= 4) && (x0 + kStrip + 4 <= g.nx);
-  const T* __restrict__ uc = reinterpret_cast<const T*>(a.u_cur);
-  const T* __restrict__ up = reinterpret_cast<const T*>(a.u_prev);
+  const T* __restrict__ uc = after_wait(reinterpret_cast<const T*>(a.u_cur));
+  const T* __restrict__ up = after_wait(reinterpret_cast<const T*>(a.u_prev));
 
   // Own row (mirrored if it lies beyond ny, zero if not needed).
   const bool row_valid = y < g.ny;
@@ -238,18 +240,18 @@ static cudaError_t launch_vel(const StepArgs& a, cudaStream_t s) {
     const int64_t nyb = (g.ny + a.zblock - 1) / a.zblock;
     const int64_t warps = nstrips * nyb;
     const int64_t blocks = (warps + kWarps2D - 1) / kWarps2D;
-    step2d_velocity_kernel<R, T, kWarps2D><<<(unsigned)blocks, kWarps2D * 32, 0, s>>>(a);
+    count_launch();
+    return launch_chained(step2d_velocity_kernel<R, T, kWarps2D>, (unsigned)blocks, kWarps2D * 32, 0, s, a);
   } else {
     dim3 grid((unsigned)nstrips, (unsigned)((g.ny + kRows3D - 1) / kRows3D),
               (unsigned)((g.nz + a.zblock - 1) / a.zblock));
     if constexpr (sizeof(T) == 4) {
       return launch_step3d_ring(a, 2 * R, s);
     } else {
-      step3d_velocity_kernel<R, T, kRows3D><<<grid, kRows3D * 32, 0, s>>>(a);
+      count_launch();
+      return launch_chained(step3d_velocity_kernel<R, T, kRows3D>, grid, kRows3D * 32, 0, s, a);
     }
   }
-  count_launch();
-  return cudaGetLastError();
 }
 
 template <typename T>

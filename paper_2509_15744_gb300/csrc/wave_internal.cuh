@@ -111,6 +111,40 @@ __device__ __forceinline__ float f4_get(const float4& v, int i) {
   return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
 }
 
+// ---- chained launches ---------------------------------------------------------
+// The kernels of a time loop (step, source / receiver, step, ...) are launched
+// as programmatic dependents: the next one's CTAs start while the last ones of
+// this one finish, which hides the launch latency of small grids.  Every such
+// kernel begins with chain_wait(): it lets its own successor start and returns
+// when all work before it in the stream is complete and visible.  Pointers to
+// what earlier launches wrote go through after_wait(), so that no read-only
+// (invariant) load of them can be moved above the wait.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename P>
+__device__ __forceinline__ P* after_wait(P* p) {
+  asm volatile("" : "+l"(p));
+  return p;
+}
+template <typename Arg>
+inline cudaError_t launch_chained(void (*kernel)(Arg), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                  const Arg& arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, arg);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // ---- step kernel arguments ----------------------------------------------
 // One leapfrog step u_next = 2 u_cur - u_prev + coef * (h^2 L u_cur), written
 // over u_prev, with the sensitivity increment acc += acc_scale * c where
