@@ -182,6 +182,11 @@ step3d_velocity_pair_kernel(BatchArgs b) {
       }
     }
   }
+  const bool yplain = ty0 >= R && ty0 + TY + R <= g.ny;   // uniform
+  const int nz_plain = min(zs_end, (int)g.nz);
+  const uint32_t d0 = 4u * (uint32_t)s_dst[0], d1 = 4u * (uint32_t)s_dst[PT::K - 1];
+  const bool has1 = PT::K > 1 && tid + (PT::K - 1) * PT::NT < PT::ROWS * PT::CH;
+  static_assert(PT::K <= 2 && PT::NT <= PT::ROWS * PT::CH, "at most two chunks per thread, the first one always");
   // x ghosts of a ragged own row (nx not a multiple of the strip): lanes
   // 0..r-1 (left end) and 8..8+r-1 (right end) write the mirror values into
   // the staged row; computed where used, so that grids whose rows end on strip
@@ -244,8 +249,22 @@ step3d_velocity_pair_kernel(BatchArgs b) {
     // (the wall plane of a Dirichlet box as zeros; the planes behind it
     // negated, copied by hand: the top r planes of the grid only), so the
     // stencil reads every staged plane as it is.
+    const float* sA = ucA + (int64_t)z0 * g.plane;   // plane p of the next call
+    const float* sB = ucB + (int64_t)z0 * g.plane;
     auto stage = [&](int p, int buf) {
-      if (p < zs_end) {
+      // Most planes of most CTAs mirror nothing: copies from a running pointer,
+      // without the masks (512^3 x 8 shots 3068 -> 3020 us a launch, 1024^3 x 4
+      // with compensation 14.79 -> 14.25 ms).
+      if (yplain && p < nz_plain) {
+        const uint32_t sb = smem0 + (uint32_t)(buf * PT::TILE) * 4u;
+        constexpr uint32_t fB = (uint32_t)(NB * PT::TILE) * 4u;
+        pcp16(sb + d0, sA + c_off[0], c_sz[0]);
+        if (has1) pcp16(sb + d1, sA + c_off[PT::K - 1], c_sz[PT::K - 1]);
+        if (two) {
+          pcp16(sb + fB + d0, sB + c_off[0], c_sz[0]);
+          if (has1) pcp16(sb + fB + d1, sB + c_off[PT::K - 1], c_sz[PT::K - 1]);
+        }
+      } else if (p < zs_end) {
         float zsg = 1.f;
         const int64_t ps = p < g.nz ? p : mirror_index(p, g.nz, g.bc, &zsg);
         const uint32_t zmask = zsg != 0.f ? 0xffffffffu : 0u;   // 0: zero-fill every chunk
@@ -279,6 +298,8 @@ step3d_velocity_pair_kernel(BatchArgs b) {
           }
         }
       }
+      sA += g.plane;
+      sB += g.plane;
       pcp_commit();
     };
 
