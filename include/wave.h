@@ -140,11 +140,12 @@ typedef struct {
   double forward_ms;    /* device time of the forward pass(es), misfit and k included */
   double adjoint_ms;    /* device time of the superposed / adjoint pass(es) and the finish */
   double total_ms;      /* device time of the whole call */
-  double step_bytes;    /* algorithmic bytes of the step-kernel launches (per cell and launch:
+  double step_bytes;    /* algorithmic bytes of the steps (per cell and step:
                            read u^n, u^{n-1}, coef [, b], write u^{n+1} per field, accumulator
                            [+ compensation] read-modify-write once) */
   double cell_updates;  /* sum over shots of cells x N_s: the gradient cell-updates of the call */
-  int64_t step_launches;
+  int64_t step_launches; /* steps; a launch that takes several steps, or two fields that were advanced by a
+                           launch each, counts each of them */
 } wave_gradient_metrics;
 
 typedef struct wave_model_s* wave_model;
@@ -161,7 +162,8 @@ uint64_t wave_launch_count(void);
  * events on its stream.  wave_timing_read waits for the recorded events and
  * returns the summed kernel time, the number of timed launches and their
  * algorithmic bytes (per cell: read u^n, u^{n-1}, coef [+ b], write u^{n+1},
- * [+ accumulator RMW, + compensation RMW]).  Enabling resets the counters.
+ * [+ accumulator RMW, + compensation RMW]).  A launch that takes several 2D
+ * steps counts every step.  Enabling resets the counters.
  * The events are recorded as external events (cudaEventRecordExternal): a
  * call captured into a CUDA graph while timing is enabled records them at
  * each replay, and wave_timing_read then returns the last replay's kernel
@@ -198,8 +200,10 @@ wave_status wave_model_create(const wave_grid_desc* desc, const float* param_dev
                               wave_model* out);
 wave_status wave_model_destroy(wave_model model);
 /* Tuning hook (used by the autotuner): the number of rows (2D) or planes (3D)
- * that one warp (2D) or CTA (3D) of the step kernel marches over.  Any value
- * >= 1 is valid; it changes speed, never results. */
+ * that one warp (2D) or CTA (3D) of the one-step kernels marches over; the
+ * default follows the grid, so that small grids fill the chip.  Any value >= 1
+ * is valid; it changes speed, never results.  The time loops that take several
+ * 2D steps per launch have their own split. */
 wave_status wave_model_set_block(wave_model model, int64_t zblock);
 wave_status wave_model_get_block(wave_model model, int64_t* zblock);
 /* Full tiling of the 3D FP32 step kernel: zblock as above, tile_rows (8 or 16
@@ -272,7 +276,11 @@ wave_status wave_step(wave_model model, int32_t nfields, const void* const* cur_
  * Leapfrog u^{n+1} = 2u^n - u^{n-1} + dt^2/a (L u^n + f^n) for n = 1..N_s with
  * traces of levels 0..N_s written to each shot's traces_dev.
  * init_dev: NULL for u^0 = u^1 = 0 (Eq. IC), else dense {u^0, u^1} (2 grids).
- * final_dev: NULL, or dense output {u^N, u^{N+1}} of the last shot. */
+ * final_dev: NULL, or dense output {u^N, u^{N+1}} of the last shot.
+ * 2D grids of FP32 storage with nx >= 128, ny >= 16 and at most 2^29 cells
+ * advance several steps per launch, from one pair of level grids to another
+ * (two grids more workspace per field); so do the passes of wave_adjoint_
+ * sensitivity there, except WAVE_EXACT_STORED. */
 wave_status wave_forward_workspace_size(wave_model model, const wave_shot* shots, int32_t nshots,
                                         size_t* bytes);
 wave_status wave_forward(wave_model model, const wave_shot* shots, int32_t nshots,
