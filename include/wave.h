@@ -277,7 +277,7 @@ wave_status wave_step(wave_model model, int32_t nfields, const void* const* cur_
  * traces of levels 0..N_s written to each shot's traces_dev.
  * init_dev: NULL for u^0 = u^1 = 0 (Eq. IC), else dense {u^0, u^1} (2 grids).
  * final_dev: NULL, or dense output {u^N, u^{N+1}} of the last shot.
- * 2D grids of FP32 storage with nx >= 128, ny >= 16 and at most 2^29 cells
+ * 2D grids of FP32 storage with nx >= 128, ny >= 16 and at most 2^32 cells
  * advance several steps per launch, from one pair of level grids to another
  * (two grids more workspace per field); so do the passes of wave_adjoint_
  * sensitivity there, except WAVE_EXACT_STORED. */

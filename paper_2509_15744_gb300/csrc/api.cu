@@ -526,13 +526,14 @@ struct TileWs {
 // idle), a large one shallow ones.  Measured at the fits' choices and next to
 // them, 251^2 order 2, 6400 steps: 2 rows S = 12 5.1 ms (8: 5.6, 4: 7.6), 4 rows
 // S = 24 6.8; 2048^2 order 8, 800 steps: 4 rows S = 3 16.4 ms (2: 19.1).
-// Grids below 128 cells in x or 16 in y, above 2^29 cells (the second pair of
-// levels costs 2 grids) and the other storage types keep one step per launch.
+// Grids below 128 cells in x or 16 in y, above 2^32 cells (the second pair of
+// levels costs 2 grids, 34 GB there) and the other storage types keep one step
+// per launch.
 static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, Tile2DPlan* out, int64_t* entries) {
   const Geom& g = m->g;
   if (m->d.ndim != 2 || m->d.storage != WAVE_F32) return false;
   const bool tmem = m->d.physics == WAVE_DENSITY || nfields == 2;   // the tensor-memory kernel has 4 rows per warp
-  if (g.nx < kStrip || g.ny < 16 || g.cells > ((int64_t)1 << 29)) return false;
+  if (g.nx < kStrip || g.ny < 16 || g.cells > ((int64_t)1 << 32)) return false;
   const int nx = (int)g.nx, ny = (int)g.ny, r = g.r;
   double best = 0.0;
   bool found = false;
