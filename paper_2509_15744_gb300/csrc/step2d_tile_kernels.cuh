@@ -591,13 +591,19 @@ __global__ void __launch_bounds__(512, 1) tile2d_tmem_kernel(Tile2DArgs a) {
         u1[f][i] = rg.load<nc>(a.cur[f], off0 + i * a.g.px);
       }
   };
-  let_next_start();
   if (!a.overlap) load_levels(std::true_type());
   if (R > 2) clear_spare(share, NF * 2 * rh);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   Points<RB, NF> pts;
   pts.init(a, rg, s_flag, r0, force);   // CTA barriers: the allocation is visible after them
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  // Only now, when every CTA of this launch holds its tensor memory, may the
+  // next launch start.  Its CTAs allocate before they wait for this launch: on
+  // an SM that CTAs of several launches share (regions of few rows), one that
+  // came before a CTA of this launch had its columns could take them and wait
+  // for the CTA that then never gets any.  This way what a CTA waits for,
+  // columns or a launch, is always held or run by CTAs that have their columns.
+  let_next_start();
   const uint32_t tm_base = s_tm;
   const uint32_t tm = tm_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * kCols);
   auto col = [&](int q, int i) -> uint32_t { return tm + (uint32_t)((q * RB + i) * 4); };
