@@ -280,9 +280,16 @@ wave_status wave_step(wave_model model, int32_t nfields, const void* const* cur_
  * 2D grids of FP32 storage with nx >= 128, ny >= 16 and at most 2^32 cells
  * advance several steps per launch, from one pair of level grids to another
  * (two grids more workspace per field); so do the passes of wave_adjoint_
- * sensitivity there, except WAVE_EXACT_STORED. */
+ * sensitivity there, except WAVE_EXACT_STORED.
+ * *_workspace_size returns the size with which a call runs fastest,
+ * *_workspace_min the least it accepts.  They differ for those grids only:
+ * with a workspace below *_workspace_size the call takes one step per launch,
+ * with the same results.  Calls with less than *_workspace_min return
+ * WAVE_EWORKSPACE. */
 wave_status wave_forward_workspace_size(wave_model model, const wave_shot* shots, int32_t nshots,
                                         size_t* bytes);
+wave_status wave_forward_workspace_min(wave_model model, const wave_shot* shots, int32_t nshots,
+                                       size_t* bytes);
 wave_status wave_forward(wave_model model, const wave_shot* shots, int32_t nshots,
                          const float* init_dev, float* final_dev,
                          void* workspace_dev, size_t ws_bytes, void* stream);
@@ -311,6 +318,8 @@ wave_status wave_forward(wave_model model, const wave_shot* shots, int32_t nshot
  * (u^j - u^{j-1}); k_dev receives 0.  Neither new mode supports batched = 1. */
 wave_status wave_gradient_workspace_size(wave_model model, const wave_shot* shots, int32_t nshots,
                                          const wave_gradient_opts* opts, size_t* bytes);
+wave_status wave_gradient_workspace_min(wave_model model, const wave_shot* shots, int32_t nshots,
+                                        const wave_gradient_opts* opts, size_t* bytes);
 wave_status wave_adjoint_sensitivity(wave_model model, const wave_shot* shots, int32_t nshots,
                                      const wave_gradient_opts* opts, float* grad_dev,
                                      double* misfit_dev, double* k_dev, double* grad_norm_dev,

@@ -834,8 +834,9 @@ extern "C" wave_status wave_step(wave_model m, int32_t nfields, const void* cons
 // ---------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------
-static void carve_forward(Carve& c, const wave_model_s* m, const wave_shot* shots, int32_t nshots, void** u0,
-                          void** u1, int64_t** recp, TileWs* tw) {
+// tiles: with the buffers of the several-steps path, where the grid has one
+static void carve_forward(Carve& c, const wave_model_s* m, const wave_shot* shots, int32_t nshots, bool tiles,
+                          void** u0, void** u1, int64_t** recp, TileWs* tw) {
   int32_t maxrec = 1;
   for (int s = 0; s < nshots; ++s) maxrec = std::max(maxrec, shots[s].nrec);
   const size_t eb = storage_bytes(m->d.storage);
@@ -843,11 +844,10 @@ static void carve_forward(Carve& c, const wave_model_s* m, const wave_shot* shot
   *u1 = c.take_bytes(m->g.cells * eb);
   *recp = c.take<int64_t>(maxrec);
   void* const u[2] = {*u0, *u1};
-  carve_tile(c, m, maxrec, 1, u, tw);
+  if (tiles) carve_tile(c, m, maxrec, 1, u, tw);
 }
 
-extern "C" wave_status wave_forward_workspace_size(wave_model m, const wave_shot* shots, int32_t nshots,
-                                                   size_t* bytes) {
+static wave_status forward_bytes(wave_model m, const wave_shot* shots, int32_t nshots, bool tiles, size_t* bytes) {
   if (!m || !bytes) return WAVE_EINVAL;
   wave_status st = validate_shots(m, shots, nshots, false);
   if (st != WAVE_OK) return st;
@@ -855,9 +855,17 @@ extern "C" wave_status wave_forward_workspace_size(wave_model m, const wave_shot
   void *u0, *u1;
   int64_t* recp;
   TileWs tw;
-  carve_forward(c, m, shots, nshots, &u0, &u1, &recp, &tw);
+  carve_forward(c, m, shots, nshots, tiles, &u0, &u1, &recp, &tw);
   *bytes = c.off;
   return WAVE_OK;
+}
+extern "C" wave_status wave_forward_workspace_size(wave_model m, const wave_shot* shots, int32_t nshots,
+                                                   size_t* bytes) {
+  return forward_bytes(m, shots, nshots, true, bytes);
+}
+extern "C" wave_status wave_forward_workspace_min(wave_model m, const wave_shot* shots, int32_t nshots,
+                                                  size_t* bytes) {
+  return forward_bytes(m, shots, nshots, false, bytes);
 }
 
 extern "C" wave_status wave_forward(wave_model m, const wave_shot* shots, int32_t nshots, const float* init_dev,
@@ -865,8 +873,9 @@ extern "C" wave_status wave_forward(wave_model m, const wave_shot* shots, int32_
   if (!m) return WAVE_EINVAL;
   wave_status st = validate_shots(m, shots, nshots, true);
   if (st != WAVE_OK) return st;
-  size_t need = 0;
-  wave_forward_workspace_size(m, shots, nshots, &need);
+  size_t need = 0, full = 0;
+  forward_bytes(m, shots, nshots, false, &need);
+  forward_bytes(m, shots, nshots, true, &full);
   if (!ws || ws_bytes < need || reinterpret_cast<uintptr_t>(ws) % 256) return WAVE_EWORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   const Geom& g = m->g;
@@ -876,7 +885,7 @@ extern "C" wave_status wave_forward(wave_model m, const wave_shot* shots, int32_
   void *ua, *ub;
   int64_t* recp;
   TileWs tw;
-  carve_forward(c, m, shots, nshots, &ua, &ub, &recp, &tw);
+  carve_forward(c, m, shots, nshots, ws_bytes >= full, &ua, &ub, &recp, &tw);
   const int64_t ncells = g.nx * g.ny * g.nz;
   for (int si = 0; si < nshots; ++si) {
     const wave_shot& sh = shots[si];
@@ -956,7 +965,7 @@ struct GradWs {
 };
 
 static void carve_gradient(Carve& c, const wave_model_s* m, const wave_shot* shots, int32_t nshots, int mode,
-                           GradWs* w) {
+                           bool tiles, GradWs* w) {
   int64_t maxres = 1;
   int32_t maxrec = 1;
   for (int s = 0; s < nshots; ++s) {
@@ -976,7 +985,7 @@ static void carve_gradient(Carve& c, const wave_model_s* m, const wave_shot* sho
   w->parts = c.take<double>(1024);
   w->scal = c.take<double>(8);
   void* const u[4] = {w->u0, w->u1, w->u2, w->u3};
-  carve_tile(c, m, maxrec, two ? 2 : 1, u, &w->tile);
+  if (tiles) carve_tile(c, m, maxrec, two ? 2 : 1, u, &w->tile);
 }
 
 static wave_status validate_opts(const wave_model_s* m, const wave_gradient_opts* o) {
@@ -1068,8 +1077,8 @@ static void carve_exact(Carve& c, const wave_model_s* m, const wave_shot* shots,
   w->scal = c.take<double>(8);
 }
 
-extern "C" wave_status wave_gradient_workspace_size(wave_model m, const wave_shot* shots, int32_t nshots,
-                                                    const wave_gradient_opts* opts, size_t* bytes) {
+static wave_status gradient_bytes(wave_model m, const wave_shot* shots, int32_t nshots,
+                                  const wave_gradient_opts* opts, bool tiles, size_t* bytes) {
   if (!m || !bytes) return WAVE_EINVAL;
   wave_status st = validate_shots(m, shots, nshots, false);
   if (st != WAVE_OK) return st;
@@ -1084,12 +1093,19 @@ extern "C" wave_status wave_gradient_workspace_size(wave_model m, const wave_sho
     carve_batched(c, m, shots, nshots, &w);
   } else {
     GradWs w;
-    carve_gradient(c, m, shots, nshots, opts->mode, &w);
+    carve_gradient(c, m, shots, nshots, opts->mode, tiles, &w);
   }
   *bytes = c.off;
   return WAVE_OK;
 }
-
+extern "C" wave_status wave_gradient_workspace_size(wave_model m, const wave_shot* shots, int32_t nshots,
+                                                    const wave_gradient_opts* opts, size_t* bytes) {
+  return gradient_bytes(m, shots, nshots, opts, true, bytes);
+}
+extern "C" wave_status wave_gradient_workspace_min(wave_model m, const wave_shot* shots, int32_t nshots,
+                                                   const wave_gradient_opts* opts, size_t* bytes) {
+  return gradient_bytes(m, shots, nshots, opts, false, bytes);
+}
 
 // Final scaling into grad_dev with the FP64 2-norm of the result (Sec. 4's
 // K~, or the exact gradient), and the call's scalars for the metrics.
@@ -1389,8 +1405,9 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
   st = validate_opts(m, opts);
   if (st != WAVE_OK) return st;
   if (opts->objective == WAVE_OBJ_PATCH && !(opts->patch_sign == 1.0 || opts->patch_sign == -1.0)) return WAVE_EINVAL;
-  size_t need = 0;
-  wave_gradient_workspace_size(m, shots, nshots, opts, &need);
+  size_t need = 0, full = 0;
+  gradient_bytes(m, shots, nshots, opts, false, &need);
+  gradient_bytes(m, shots, nshots, opts, true, &full);
   if (!ws || ws_bytes < need || reinterpret_cast<uintptr_t>(ws) % 256) return WAVE_EWORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   if (opts->mode == WAVE_EXACT_STORED)
@@ -1402,7 +1419,7 @@ extern "C" wave_status wave_adjoint_sensitivity(wave_model m, const wave_shot* s
   const double dt = m->d.dt;
   Carve c(ws);
   GradWs w;
-  carve_gradient(c, m, shots, nshots, opts->mode, &w);
+  carve_gradient(c, m, shots, nshots, opts->mode, ws_bytes >= full, &w);
   double* kd = w.scal + 0;
   double* misfit_acc = misfit_dev ? misfit_dev : w.scal + 3;
   const bool sym = opts->mode == WAVE_SYMMETRIC_K;

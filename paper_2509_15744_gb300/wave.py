@@ -82,9 +82,12 @@ _model_set_debug = _sig("wave_model_set_debug", _st, _vp, _i32, C.c_int64)
 _model_pitch = _sig("wave_model_pitch", _st, _vp, C.POINTER(C.c_int64))
 _step = _sig("wave_step", _st, _vp, _i32, C.POINTER(_vp), C.POINTER(_vp), C.POINTER(C.c_float), _vp, _vp, _vp)
 _fwd_ws = _sig("wave_forward_workspace_size", _st, _vp, C.POINTER(ShotDesc), _i32, C.POINTER(_sz))
+_fwd_min = _sig("wave_forward_workspace_min", _st, _vp, C.POINTER(ShotDesc), _i32, C.POINTER(_sz))
 _forward = _sig("wave_forward", _st, _vp, C.POINTER(ShotDesc), _i32, _vp, _vp, _vp, _sz, _vp)
 _grad_ws = _sig("wave_gradient_workspace_size", _st, _vp, C.POINTER(ShotDesc), _i32, C.POINTER(GradOpts),
                 C.POINTER(_sz))
+_grad_min = _sig("wave_gradient_workspace_min", _st, _vp, C.POINTER(ShotDesc), _i32, C.POINTER(GradOpts),
+                 C.POINTER(_sz))
 _adjoint_sensitivity = _sig("wave_adjoint_sensitivity", _st, _vp, C.POINTER(ShotDesc), _i32, C.POINTER(GradOpts),
                             _vp, _vp, _vp, _vp, _vp, _sz, _vp)
 
@@ -257,6 +260,7 @@ class Model:
         self._h = h_
         self._fws = None
         self._gws = None
+        self._denied = {}       # workspace sizes that did not fit the device
         self.grad_norm = None   # device FP64 ||grad||_2 of the last gradient call
 
     def __del__(self):
@@ -347,12 +351,25 @@ class Model:
         sg = (C.c_float * n)(*[float(v) for v in acc_sign]) if acc_sign is not None else None
         _check(_step(self._h, n, ca, pa, sg, _ptr(acc), _ptr(comp), _stream(stream)), "wave_step")
 
-    def _ensure(self, attr, nbytes):
+    def _ensure(self, attr, nbytes, least):
+        """The kept workspace of at least nbytes; of at least `least` bytes
+        where nbytes did not fit the device (2D: one step per launch then)."""
         ws = getattr(self, attr)
-        if ws is None or ws.numel() < nbytes:
-            ws = _workspace(nbytes, self.param.device)
-            setattr(self, attr, ws)
-        return ws
+        if ws is not None and ws.numel() >= nbytes:
+            return ws
+        if nbytes < self._denied.get(attr, nbytes + 1):
+            try:
+                ws = _workspace(nbytes, self.param.device)
+            except torch.OutOfMemoryError:
+                if least >= nbytes:
+                    raise
+                self._denied[attr] = nbytes   # not tried again on every call
+            else:
+                setattr(self, attr, ws)
+                return ws
+        if ws is None or ws.numel() < least:
+            setattr(self, attr, _workspace(least, self.param.device))
+        return getattr(self, attr)
 
     def forward(self, shots: Sequence[Shot], init: Optional[torch.Tensor] = None, return_final: bool = False,
                 stream=None):
@@ -361,14 +378,15 @@ class Model:
         dev = self.param.device
         traces = [torch.empty((s.nrec, s.nt + 1), dtype=torch.float32, device=dev) for s in shots]
         arr = _shot_descs(shots, traces)
-        nbytes = _sz(0)
+        nbytes, least = _sz(0), _sz(0)
         _check(_fwd_ws(self._h, arr, len(shots), C.byref(nbytes)), "wave_forward_workspace_size")
-        ws = self._ensure("_fws", nbytes.value)
+        _check(_fwd_min(self._h, arr, len(shots), C.byref(least)), "wave_forward_workspace_min")
         final = torch.empty((2,) + self.shape, dtype=torch.float32, device=dev) if return_final else None
         if init is not None:
             init = init.contiguous().to(torch.float32)
             if tuple(init.shape) != (2,) + self.shape:
                 raise ValueError("init must be [2, *shape]")
+        ws = self._ensure("_fws", nbytes.value, least.value)   # after the outputs: it can do with less
         _check(_forward(self._h, arr, len(shots), _ptr(init), _ptr(final), _ptr(ws), ws.numel(), _stream(stream)),
                "wave_forward")
         return (traces, final) if return_final else traces
@@ -391,13 +409,14 @@ class Model:
         o.k = float(k) if k is not None else 0.0
         o.k_ratio = float(k_ratio) if k_ratio is not None else 0.0
         arr = _shot_descs(shots)
-        nbytes = _sz(0)
+        nbytes, least = _sz(0), _sz(0)
         _check(_grad_ws(self._h, arr, len(shots), C.byref(o), C.byref(nbytes)), "wave_gradient_workspace_size")
-        ws = self._ensure("_gws", nbytes.value)
+        _check(_grad_min(self._h, arr, len(shots), C.byref(o), C.byref(least)), "wave_gradient_workspace_min")
         grad = out if out is not None else torch.empty(self.shape, dtype=torch.float32, device=dev)
         mis = torch.empty(1, dtype=torch.float64, device=dev)
         kd = torch.empty(1, dtype=torch.float64, device=dev)
         norm = torch.empty(1, dtype=torch.float64, device=dev)
+        ws = self._ensure("_gws", nbytes.value, least.value)   # after the outputs: it can do with less
         _check(_adjoint_sensitivity(self._h, arr, len(shots), C.byref(o), _ptr(grad), _ptr(mis), _ptr(kd),
                                     _ptr(norm), _ptr(ws), ws.numel(), _stream(stream)), "wave_adjoint_sensitivity")
         self.grad_norm = norm
