@@ -129,16 +129,22 @@ step2d_velocity_kernel(StepArgs a) {
 // ---------------------------------------------------------------------------
 // 3D: CTA of TY rows x 128 cells, march in z (2.5D)
 // ---------------------------------------------------------------------------
-// Four CTAs per SM: this kernel hides its load latency with other CTAs, not by
-// staging ahead.  Orders 6 and 8 take 97 and 122 registers unbounded (2 CTAs);
-// held to 64 a step of 300 x 311 x 333, order 8, BF16 storage takes 204 us
-// instead of 273.  Orders 2 and 4 need no more than 64 by themselves.
-template <int R, typename T, int TY>
-__global__ void __launch_bounds__(TY * 32, R >= 3 ? 4 : 1)
+// 16-bit storage.  This kernel hides its load latency with other CTAs, not by
+// staging ahead: CTAS = 4 per SM where the grid has that many.  Orders 6 and 8
+// take 97 and 122 registers by themselves (CTAS = 0; two CTAs per SM) and spill
+// when held to 64: that pays only where the third and fourth CTA exist (a forward
+// step of order 8, BF16: 320 x 300 x 128, 380 CTAs, 126 us by itself and 105 held;
+// 320 x 230 x 128, 290 CTAs, 64 and 79).  Orders 2 and 4 need no more than 64
+// and are not held: asked for less than four CTAs, ptxas takes 96 and 120.
+// Launched plainly, not chained: the CTAs of a chained launch are placed while
+// the last ones of the launch before still run, unevenly over the SMs, and
+// march for the whole kernel where they are (order 2, 40 x 300 x 384, 16-step
+// gradient: 2.0 ms chained, 1.65 plain).
+template <int R, typename T, int TY, int CTAS>
+__global__ void __launch_bounds__(TY * 32, CTAS)
 step3d_velocity_kernel(StepArgs a) {
   static_assert(TY >= 2 * R, "the first 2r warps stage the y halo rows");
   __shared__ __align__(16) float sm[2][TY + 2 * R][kRowW];
-  chain_wait();
   const Geom& g = a.g;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -149,8 +155,8 @@ step3d_velocity_kernel(StepArgs a) {
   const int64_t z1 = min(z0 + a.zblock, g.nz);
   const int64_t xl = x0 + 4 * lane;
   const bool xin = (x0 >= 4) && (x0 + kStrip + 4 <= g.nx);
-  const T* __restrict__ uc = after_wait(reinterpret_cast<const T*>(a.u_cur));
-  const T* __restrict__ up = after_wait(reinterpret_cast<const T*>(a.u_prev));
+  const T* __restrict__ uc = reinterpret_cast<const T*>(a.u_cur);
+  const T* __restrict__ up = reinterpret_cast<const T*>(a.u_prev);
 
   // Own row (mirrored if it lies beyond ny, zero if not needed).
   const bool row_valid = y < g.ny;
@@ -249,7 +255,14 @@ static cudaError_t launch_vel(const StepArgs& a, cudaStream_t s) {
       return launch_step3d_ring(a, 2 * R, s);
     } else {
       count_launch();
-      return launch_chained(step3d_velocity_kernel<R, T, kRows3D>, grid, kRows3D * 32, 0, s, a);
+      // more full z-blocks than two CTAs per SM take at once (the last block of a
+      // column counts by its planes: 33 x 500 x 384, order 8, 378 CTAs of which
+      // half have one plane, takes 1.40 ms by itself and 1.80 held)
+      if (R >= 3 && (int64_t)grid.x * grid.y * g.nz > 2 * 152 * a.zblock)
+        step3d_velocity_kernel<R, T, kRows3D, R >= 3 ? 4 : 0><<<grid, kRows3D * 32, 0, s>>>(a);
+      else
+        step3d_velocity_kernel<R, T, kRows3D, 0><<<grid, kRows3D * 32, 0, s>>>(a);
+      return cudaGetLastError();
     }
   }
 }
