@@ -280,7 +280,10 @@ wave_status wave_step(wave_model model, int32_t nfields, const void* const* cur_
  * 2D grids of FP32 storage with nx >= 128, ny >= 16 and at most 2^32 cells
  * advance several steps per launch, from one pair of level grids to another
  * (two grids more workspace per field); so do the passes of wave_adjoint_
- * sensitivity there, except WAVE_EXACT_STORED.
+ * sensitivity there, except WAVE_EXACT_STORED.  One step per launch is kept by
+ * grids of order 6 with fewer than 26 rows (28 with two fields) unless their
+ * number is even (a multiple of 4), by records of one or two steps (velocity
+ * form) and where receivers take a large part of the cells.
  * *_workspace_size returns the size with which a call runs fastest,
  * *_workspace_min the least it accepts.  They differ for those grids only:
  * with a workspace below *_workspace_size the call takes one step per launch,

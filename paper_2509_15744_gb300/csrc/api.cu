@@ -515,6 +515,30 @@ struct TileWs {
   int64_t entries = 0;
 };
 
+// Whether several steps per launch pay for the records at hand.  Records of one
+// or two steps do not earn back the lists (251^2, order 2, a forward of one step: 77
+// us, 58 with a launch per step; density form 99, 70; its two-field mode
+// gains from two steps on).  Where receivers fill whole
+// regions, those regions record and inject for every other one's time, while
+// the one-step kernels spread that over the chip; velocity form, several waves
+// of regions, several steps against one step, ms:
+//   2048^2 order 2, 200 steps, gradient: receivers in 0.375 of the cells 18.1, 21.2;
+//   in 0.75 33.5, 32.9;  order 8: 0.25 20.6, 23.4; 0.375 27.1, 27.4; 0.75 47.6, 39.2;
+//   two fields, 1500^2 order 8: 0.094 11.1, 11.3; 0.19 13.3, 12.7; 0.375 20.5, 17.9.
+// A record of a few steps pays for the lists in addition (2048^2 order 8, 4 steps:
+// 0.023 of the cells 0.40, 0.39; 0.19 0.58, 0.47; in one wave 512^2 order 4: 0.19
+// 0.22, 0.23; 0.75 0.24, 0.23).  The density form gains throughout (2048^2, 100
+// steps, 0.6: 15.0, 22.9; 4 steps: 1.00, 0.91).
+static bool tile2d_pays(const wave_model_s* m, const Tile2DPlan& p, int nfields, int32_t maxrec, int32_t maxnt) {
+  const double f = (double)maxrec / ((double)m->g.nx * (double)m->g.ny);
+  const bool density = m->d.physics == WAVE_DENSITY;
+  if (maxnt < (density && nfields == 2 ? 2 : 3)) return false;
+  if (density) return maxnt >= 16 || f <= 0.5;
+  const bool waves = (int64_t)p.nkx * p.nky > 152;
+  if (maxnt < 16) return f <= (!waves ? 1.0 / 4 : m->g.r <= 2 ? 1.0 / 32 : 1.0 / 64);
+  return !waves || f <= (m->g.r <= 2 ? 1.0 / 2 : nfields == 1 ? 1.0 / 3 : 1.0 / 8);
+}
+
 // Region split for the model's 2D grid: rows per warp (2 or 4; 16 warps) and
 // steps per launch S with the least modelled time of a step.  The figures are
 // fits to measured gradient calls on GB300 (128^2, 251^2, 363^2, 2048^2, 6001 x
@@ -528,8 +552,11 @@ struct TileWs {
 // S = 24 6.8; 2048^2 order 8, 800 steps: 4 rows S = 3 16.4 ms (2: 19.1).
 // Grids below 128 cells in x or 16 in y, above 2^32 cells (the second pair of
 // levels costs 2 grids, 34 GB there) and the other storage types keep one step
-// per launch.
-static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, Tile2DPlan* out, int64_t* entries) {
+// per launch; so do grids that no split fits (order 6 needs h = 12, so fewer than
+// 26 rows, or 28 with two fields, must be one region), and calls that several steps would slow down
+// (tile2d_pays).
+static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, int32_t maxnt, Tile2DPlan* out,
+                        int64_t* entries) {
   const Geom& g = m->g;
   if (m->d.ndim != 2 || m->d.storage != WAVE_F32) return false;
   const bool tmem = m->d.physics == WAVE_DENSITY || nfields == 2;   // the tensor-memory kernel has 4 rows per warp
@@ -565,7 +592,7 @@ static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, Tile
       }
     }
   }
-  if (!found) return false;
+  if (!found || !tile2d_pays(m, *out, nfields, maxrec, maxnt)) return false;
   // a cell lies in at most (w - 1) / out + 1 of the evenly placed regions of an axis, and the last one
   const int64_t bx = std::min(out->nkx, (kStrip - 1) / out->outx + 2);
   const int64_t by = std::min(out->nky, (out->rh - 1) / out->outy + 2);
@@ -574,8 +601,9 @@ static bool tile2d_plan(const wave_model_s* m, int nfields, int32_t maxrec, Tile
 }
 
 // u: the first pair of levels of each field, carved by the caller.
-static void carve_tile(Carve& c, const wave_model_s* m, int32_t maxrec, int nfields, void* const* u, TileWs* t) {
-  t->on = tile2d_plan(m, nfields, maxrec, &t->plan, &t->entries);
+static void carve_tile(Carve& c, const wave_model_s* m, int32_t maxrec, int32_t maxnt, int nfields, void* const* u,
+                       TileWs* t) {
+  t->on = tile2d_plan(m, nfields, maxrec, maxnt, &t->plan, &t->entries);
   if (!t->on) return;
   const size_t n = (size_t)t->plan.nkx * t->plan.nky;
   for (int f = 0; f < nfields; ++f)
@@ -837,14 +865,17 @@ extern "C" wave_status wave_step(wave_model m, int32_t nfields, const void* cons
 // tiles: with the buffers of the several-steps path, where the grid has one
 static void carve_forward(Carve& c, const wave_model_s* m, const wave_shot* shots, int32_t nshots, bool tiles,
                           void** u0, void** u1, int64_t** recp, TileWs* tw) {
-  int32_t maxrec = 1;
-  for (int s = 0; s < nshots; ++s) maxrec = std::max(maxrec, shots[s].nrec);
+  int32_t maxrec = 1, maxnt = 0;
+  for (int s = 0; s < nshots; ++s) {
+    maxrec = std::max(maxrec, shots[s].nrec);
+    maxnt = std::max(maxnt, shots[s].nt);
+  }
   const size_t eb = storage_bytes(m->d.storage);
   *u0 = c.take_bytes(m->g.cells * eb);
   *u1 = c.take_bytes(m->g.cells * eb);
   *recp = c.take<int64_t>(maxrec);
   void* const u[2] = {*u0, *u1};
-  if (tiles) carve_tile(c, m, maxrec, 1, u, tw);
+  if (tiles) carve_tile(c, m, maxrec, maxnt, 1, u, tw);
 }
 
 static wave_status forward_bytes(wave_model m, const wave_shot* shots, int32_t nshots, bool tiles, size_t* bytes) {
@@ -967,10 +998,11 @@ struct GradWs {
 static void carve_gradient(Carve& c, const wave_model_s* m, const wave_shot* shots, int32_t nshots, int mode,
                            bool tiles, GradWs* w) {
   int64_t maxres = 1;
-  int32_t maxrec = 1;
+  int32_t maxrec = 1, maxnt = 0;
   for (int s = 0; s < nshots; ++s) {
     maxres = std::max<int64_t>(maxres, (int64_t)(shots[s].nt + 1) * shots[s].nrec);
     maxrec = std::max(maxrec, shots[s].nrec);
+    maxnt = std::max(maxnt, shots[s].nt);
   }
   const size_t eb = storage_bytes(m->d.storage);
   w->acc = c.take<float>(m->g.cells);
@@ -985,7 +1017,7 @@ static void carve_gradient(Carve& c, const wave_model_s* m, const wave_shot* sho
   w->parts = c.take<double>(1024);
   w->scal = c.take<double>(8);
   void* const u[4] = {w->u0, w->u1, w->u2, w->u3};
-  if (tiles) carve_tile(c, m, maxrec, two ? 2 : 1, u, &w->tile);
+  if (tiles) carve_tile(c, m, maxrec, maxnt, two ? 2 : 1, u, &w->tile);
 }
 
 static wave_status validate_opts(const wave_model_s* m, const wave_gradient_opts* o) {

@@ -175,3 +175,33 @@ def test_dense_receivers_do_not_slow_the_call_down(W):
         ms[name] = min(times)
     # several steps per launch against one: 0.43 and 0.56 ms; 1.6 ms with an atomic per receiver
     assert ms["full"] < 1.25 * ms["least"], ms
+
+
+# calls that several steps per launch would slow down take one: they need no
+# second pair of level grids
+@pytest.mark.parametrize("shape,physics,order,mode,nt,dense,several", [
+    ((251, 251), "velocity", 2, "superposition", 2, 0.0, False),
+    ((251, 251), "velocity", 2, "superposition", 3, 0.0, True),
+    ((251, 251), "density", 2, "superposition", 2, 0.0, False),
+    ((251, 251), "density", 2, "symmetric", 2, 0.0, True),
+    ((300, 400), "velocity", 4, "superposition", 20, 0.8, True),      # one wave of regions
+    ((1000, 1300), "velocity", 2, "superposition", 20, 0.4, True),
+    ((1000, 1300), "velocity", 2, "superposition", 20, 0.6, False),
+    ((1000, 1300), "velocity", 8, "superposition", 20, 0.4, False),
+    ((1000, 1300), "velocity", 8, "symmetric", 20, 0.2, False),
+    ((1000, 1300), "velocity", 8, "superposition", 8, 0.1, False),
+    ((1000, 1300), "density", 2, "symmetric", 20, 0.8, True),
+    ((27, 300), "velocity", 6, "superposition", 30, 0.0, True),
+    ((25, 300), "velocity", 6, "superposition", 30, 0.0, False)])
+def test_route_of_short_records_and_dense_receivers(W, shape, physics, order, mode, nt, dense, several):
+    n = shape[0] * shape[1]
+    p = torch.full(shape, 2500.0 if physics == "velocity" else 0.5, device="cuda")
+    h, vmax = (10.0, 2500.0) if physics == "velocity" else (2e-3, 509.8366)
+    m = W.Model(p, h, O.cfl_dt(h, vmax, 2, order, 0.5), order, physics)
+    rec = torch.arange(max(4, int(dense * n)), device="cuda")
+    arr, o = W._shot_descs([W.Shot(n - 1, torch.ones(nt + 1, device="cuda"), rec)]), W.GradOpts()
+    o.mode, o.k = W.MODE[mode], 1.0
+    full, least = W._sz(0), W._sz(0)
+    assert W._grad_ws(m._h, arr, 1, W.C.byref(o), W.C.byref(full)) == 0
+    assert W._grad_min(m._h, arr, 1, W.C.byref(o), W.C.byref(least)) == 0
+    assert (full.value > least.value) == several
