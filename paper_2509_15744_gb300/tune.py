@@ -6,7 +6,9 @@ speed only, never results.  `tune()` times a short gradient call of the given
 shots with each tiling candidate in the default (plane-major) order (CUDA
 events inside libwave, `wave_timing_*`), keeps the fastest, times that tiling
 once more in the other order, applies the faster and caches the choice under
-a key of (dims, shape, order, physics, storage, Kahan, shots per launch).
+a key of (dims, shape, order, physics, storage, Kahan, shots per launch).  2D
+grids whose gradients take several steps per launch are timed by `Model.step`:
+the tiling governs the one-step kernels only.
 """
 from __future__ import annotations
 
@@ -46,8 +48,14 @@ def candidates(ndim: int, nz: int, batched: bool = False):
 
 
 def _key(model: W.Model, batch: int) -> str:
-    return json.dumps([len(model.shape), list(model.shape), model.order, model.physics, model.storage,
-                       bool(model.kahan), batch])
+    key = [len(model.shape), list(model.shape), model.order, model.physics, model.storage, bool(model.kahan), batch]
+    return json.dumps(key + ["step"] if _by_step(model) else key)
+
+
+def _by_step(model: W.Model) -> bool:
+    """The tiling has no part in this model's gradients: 2D grids that take
+    several steps per launch (wave_forward in include/wave.h)."""
+    return len(model.shape) == 2 and model.storage == "f32" and model.shape[1] >= 128 and model.shape[0] >= 16
 
 
 def _load() -> Dict[str, list]:
@@ -85,14 +93,23 @@ def tune(model: W.Model, shots: Sequence[W.Shot], steps: int = 12, batched: bool
         probe.append(W.Shot(s.src, s.wavelet[:n + 1].contiguous(), s.rec,
                             None if s.observed is None else s.observed[:, :n + 1].contiguous()))
     nz = model.shape[0]
+    if _by_step(model):
+        grids = [torch.zeros(model.pitched_shape(), device=dev) for _ in range(4 if model.kahan else 3)]
+
+        def run():
+            for i in range(steps):
+                model.step([grids[i & 1]], [grids[1 - (i & 1)]], acc=grids[2], comp=grids[3] if model.kahan else None)
+    else:
+        def run():
+            model.gradient(probe, batched=batched, k=1.0)
 
     def time_one(cand, order):
         model.set_tiling(*cand)
         model.set_schedule(order)
-        model.gradient(probe, batched=batched, k=1.0)          # warm-up (and attribute setup)
+        run()                                                  # warm-up (and attribute setup)
         torch.cuda.synchronize(dev)
         W.timing_enable(True)
-        model.gradient(probe, batched=batched, k=1.0)
+        run()
         ms, n, _ = W.timing_read()
         W.timing_enable(False)
         if verbose:
