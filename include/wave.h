@@ -323,6 +323,11 @@ wave_status wave_gradient_workspace_size(wave_model model, const wave_shot* shot
                                          const wave_gradient_opts* opts, size_t* bytes);
 wave_status wave_gradient_workspace_min(wave_model model, const wave_shot* shots, int32_t nshots,
                                         const wave_gradient_opts* opts, size_t* bytes);
+/* Steps that a launch of the call's time loops takes (the last one of a pass
+ * the rest) with a workspace of *_workspace_size bytes: 1 but for the 2D grids
+ * described at wave_forward. */
+wave_status wave_gradient_steps_per_launch(wave_model model, const wave_shot* shots, int32_t nshots,
+                                           const wave_gradient_opts* opts, int32_t* steps);
 wave_status wave_adjoint_sensitivity(wave_model model, const wave_shot* shots, int32_t nshots,
                                      const wave_gradient_opts* opts, float* grad_dev,
                                      double* misfit_dev, double* k_dev, double* grad_norm_dev,

@@ -1138,6 +1138,21 @@ extern "C" wave_status wave_gradient_workspace_min(wave_model m, const wave_shot
                                                    const wave_gradient_opts* opts, size_t* bytes) {
   return gradient_bytes(m, shots, nshots, opts, false, bytes);
 }
+extern "C" wave_status wave_gradient_steps_per_launch(wave_model m, const wave_shot* shots, int32_t nshots,
+                                                      const wave_gradient_opts* opts, int32_t* steps) {
+  if (!m || !steps) return WAVE_EINVAL;
+  wave_status st = validate_shots(m, shots, nshots, false);
+  if (st != WAVE_OK) return st;
+  st = validate_opts(m, opts);
+  if (st != WAVE_OK) return st;
+  *steps = 1;
+  if (opts->mode == WAVE_EXACT_STORED || opts->batched) return WAVE_OK;
+  Carve c(nullptr);
+  GradWs w;
+  carve_gradient(c, m, shots, nshots, opts->mode, true, &w);
+  if (w.tile.on) *steps = w.tile.plan.steps;
+  return WAVE_OK;
+}
 
 // Final scaling into grad_dev with the FP64 2-norm of the result (Sec. 4's
 // K~, or the exact gradient), and the call's scalars for the metrics.

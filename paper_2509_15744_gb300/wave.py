@@ -88,6 +88,8 @@ _grad_ws = _sig("wave_gradient_workspace_size", _st, _vp, C.POINTER(ShotDesc), _
                 C.POINTER(_sz))
 _grad_min = _sig("wave_gradient_workspace_min", _st, _vp, C.POINTER(ShotDesc), _i32, C.POINTER(GradOpts),
                  C.POINTER(_sz))
+_steps_per_launch = _sig("wave_gradient_steps_per_launch", _st, _vp, C.POINTER(ShotDesc), _i32, C.POINTER(GradOpts),
+                         C.POINTER(_i32))
 _adjoint_sensitivity = _sig("wave_adjoint_sensitivity", _st, _vp, C.POINTER(ShotDesc), _i32, C.POINTER(GradOpts),
                             _vp, _vp, _vp, _vp, _vp, _sz, _vp)
 
@@ -390,6 +392,14 @@ class Model:
         _check(_forward(self._h, arr, len(shots), _ptr(init), _ptr(final), _ptr(ws), ws.numel(), _stream(stream)),
                "wave_forward")
         return (traces, final) if return_final else traces
+
+    def steps_per_launch(self, shots: Sequence[Shot], mode: str = "superposition", batched: bool = False) -> int:
+        """Time steps that a launch takes in gradient(shots, mode=mode, batched=batched)."""
+        o, n = GradOpts(), C.c_int32(0)
+        o.mode, o.batched = MODE[mode], int(bool(batched))
+        _check(_steps_per_launch(self._h, _shot_descs(shots), len(shots), C.byref(o), C.byref(n)),
+               "wave_gradient_steps_per_launch")
+        return int(n.value)
 
     def gradient(self, shots: Sequence[Shot], objective: str = "l2", k: Optional[float] = None,
                  k_ratio: Optional[float] = None, mode: str = "superposition", batched: bool = False,
