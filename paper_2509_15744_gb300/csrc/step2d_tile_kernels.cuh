@@ -41,6 +41,7 @@
 namespace wave {
 namespace {
 
+constexpr int kTileWarps = 16;   // of a region, at most
 constexpr int kSW = kStrip + 8;   // shared row: 4 spare cells each side
 constexpr int kNoForce = 0x7fa5a5a5;   // bits of a force-plane cell without a force (a NaN no force has)
 
@@ -427,8 +428,8 @@ __device__ __forceinline__ void add_square_kahan(float sg, const float4& un, con
 }
 
 // One field.  ACC: 0 none, 1 acc, 2 with compensation; the increment's sign is SGN.
-template <int R, int RB, int NW, int ACC, int SGN>
-__global__ void __launch_bounds__(NW * 32, 1) tile2d_velocity_kernel(Tile2DArgs a) {
+template <int R, int RB, int ACC, int SGN>
+__global__ void __launch_bounds__(kTileWarps * 32, 1) tile2d_velocity_kernel(Tile2DArgs a) {
   extern __shared__ __align__(16) float smem[];
   __shared__ uint32_t s_flag[3][4];   // rows of the region with a force, with a receiver to record; [2][0]: cells taken twice
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -889,10 +890,10 @@ __global__ void __launch_bounds__(512, 1) tile2d_tmem_kernel(Tile2DArgs a) {
 }
 
 template <typename K>
-cudaError_t launch_tile(K kernel, int rb, int nw, const Tile2DArgs& a, cudaStream_t s, int per_thread = 0) {
+cudaError_t launch_tile(K kernel, int rb, const Tile2DArgs& a, cudaStream_t s, int per_thread = 0) {
   // shared bytes per region row: rows of both levels, force rows, per-thread data
   const int row = (2 * a.nfields * kSW + 2 * kStrip) * 4 + per_thread * 32 / rb;
-  cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(kernel), row * rb * nw);
+  cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(kernel), row * rb * kTileWarps);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.plan.nkx, a.plan.nky);
@@ -913,20 +914,20 @@ cudaError_t launch_tile(K kernel, int rb, int nw, const Tile2DArgs& a, cudaStrea
 
 template <int R, int RB>
 cudaError_t launch_vel(const Tile2DArgs& a, cudaStream_t s) {
-  if (!a.acc) return launch_tile(tile2d_velocity_kernel<R, RB, 16, 0, 1>, RB, 16, a, s);
+  if (!a.acc) return launch_tile(tile2d_velocity_kernel<R, RB, 0, 1>, RB, a, s);
   if (a.acc_scale > 0.f)
-    return a.comp ? launch_tile(tile2d_velocity_kernel<R, RB, 16, 2, 1>, RB, 16, a, s)
-                  : launch_tile(tile2d_velocity_kernel<R, RB, 16, 1, 1>, RB, 16, a, s);
-  return a.comp ? launch_tile(tile2d_velocity_kernel<R, RB, 16, 2, -1>, RB, 16, a, s)
-                : launch_tile(tile2d_velocity_kernel<R, RB, 16, 1, -1>, RB, 16, a, s);
+    return a.comp ? launch_tile(tile2d_velocity_kernel<R, RB, 2, 1>, RB, a, s)
+                  : launch_tile(tile2d_velocity_kernel<R, RB, 1, 1>, RB, a, s);
+  return a.comp ? launch_tile(tile2d_velocity_kernel<R, RB, 2, -1>, RB, a, s)
+                : launch_tile(tile2d_velocity_kernel<R, RB, 1, -1>, RB, a, s);
 }
 
 template <int R>
 cudaError_t launch_vel_r(const Tile2DArgs& a, cudaStream_t s) {
   if (a.nfields == 1) return a.plan.rb == 2 ? launch_vel<R, 2>(a, s) : launch_vel<R, 4>(a, s);
-  if (a.mix) return launch_tile(tile2d_tmem_kernel<R, false, 2, 3>, 4, 16, a, s);
-  return a.comp ? launch_tile(tile2d_tmem_kernel<R, false, 2, 2>, 4, 16, a, s)
-                : launch_tile(tile2d_tmem_kernel<R, false, 2, 1>, 4, 16, a, s);
+  if (a.mix) return launch_tile(tile2d_tmem_kernel<R, false, 2, 3>, 4, a, s);
+  return a.comp ? launch_tile(tile2d_tmem_kernel<R, false, 2, 2>, 4, a, s)
+                : launch_tile(tile2d_tmem_kernel<R, false, 2, 1>, 4, a, s);
 }
 
 }  // namespace

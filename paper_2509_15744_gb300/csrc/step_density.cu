@@ -541,8 +541,11 @@ static cudaError_t launch_march(const StepArgs& a, cudaStream_t s) {
   const int64_t blocks = (g.nx + kStrip - 1) / kStrip * ((g.ny + kMarchRows - 1) / kMarchRows) *
                          ((g.nz + a.zblock - 1) / a.zblock);
   const bool acc = a.acc_mass || a.acc_stiff;
+  if (NF == 2 && !acc) return cudaErrorInvalidValue;
   count_launch();
-  if (!acc) return launch_chained(step3d_density_march_kernel<NF, 0>, (unsigned)blocks, kMarchRows * 32, 0, s, a);
+  if constexpr (NF == 1) {   // two fields only advance to accumulate
+    if (!acc) return launch_chained(step3d_density_march_kernel<NF, 0>, (unsigned)blocks, kMarchRows * 32, 0, s, a);
+  }
   if (!a.comp) return launch_chained(step3d_density_march_kernel<NF, 1>, (unsigned)blocks, kMarchRows * 32, 0, s, a);
   return launch_chained(step3d_density_march_kernel<NF, 2>, (unsigned)blocks, kMarchRows * 32, 0, s, a);
 }
