@@ -22,28 +22,32 @@ __global__ void tile2d_list_kernel(Tile2DPlan P, Geom g, const int64_t* __restri
   const int y = in ? (int)(p / g.px) : 0, x = in ? (int)(p - (int64_t)y * g.px) : 0;
   const int nx = (int)g.nx, ny = (int)g.ny;
   const int ky0 = y < P.rh ? 0 : (y - P.rh) / P.outy + 1, kx0 = x < kStrip ? 0 : (x - kStrip) / P.outx + 1;
-  const int by = (P.rh - 1) / P.outy + 1, bx = (kStrip - 1) / P.outx + 1;
+  const int by = min((P.rh - 1) / P.outy + 1, P.nky - 1), bx = min((kStrip - 1) / P.outx + 1, P.nkx - 1);
   for (int iy = 0; iy <= by; ++iy) {
     const int ky = iy < by ? ky0 + iy : P.nky - 1;
     const int ys = tile_start(ky, P.nky, P.outy, ny, P.rh);
     const bool yin = in && (iy == by || ky < P.nky - 1) && y >= ys && y < ys + P.rh;
-    const bool yo = y >= tile_own_lo(ky, P.outy, P.rh, P.h) && y < tile_own_hi(ky, P.nky, P.outy, ny, P.rh, P.h);
+    if (!__any_sync(0xffffffffu, yin)) continue;
     for (int ix = 0; ix <= bx; ++ix) {
       const int kx = ix < bx ? kx0 + ix : P.nkx - 1;
       const int xs = tile_start(kx, P.nkx, P.outx, nx, kStrip);
       const bool here = yin && (ix == bx || kx < P.nkx - 1) && x >= xs && x < xs + kStrip;
-      const bool xo = x >= tile_own_lo(kx, P.outx, kStrip, P.h) && x < tile_own_hi(kx, P.nkx, P.outx, nx, kStrip, P.h);
       if (!__any_sync(0xffffffffu, here)) continue;
       const int t = here ? ky * P.nkx + kx : -1;
       const unsigned same = __match_any_sync(0xffffffffu, t);
       const int leader = __ffs(same) - 1;
+      if (count) {   // nothing waits for these
+        if (here && lane == leader) atomicAdd(count + t, __popc(same));
+        continue;
+      }
       int first = 0;
-      if (here && lane == leader) first = atomicAdd((count ? count : cursor) + t, __popc(same));
-      if (count) continue;
+      if (here && lane == leader) first = atomicAdd(cursor + t, __popc(same));
       first = __shfl_sync(0xffffffffu, first, leader) + __popc(same & ((1u << lane) - 1u));
       if (here) {
+        const bool own = y >= tile_own_lo(ky, P.outy, P.rh, P.h) && y < tile_own_hi(ky, P.nky, P.outy, ny, P.rh, P.h) &&
+                         x >= tile_own_lo(kx, P.outx, kStrip, P.h) && x < tile_own_hi(kx, P.nkx, P.outx, nx, kStrip, P.h);
         const int pos = (y - ys) * kStrip + (x - xs);
-        ent[first] = make_int2(pos | (yo && xo ? (int)0x80000000 : 0), r);
+        ent[first] = make_int2(pos | (own ? (int)0x80000000 : 0), r);
       }
     }
   }
