@@ -354,8 +354,8 @@ class Model:
         _check(_step(self._h, n, ca, pa, sg, _ptr(acc), _ptr(comp), _stream(stream)), "wave_step")
 
     def _ensure(self, attr, nbytes, least):
-        """The kept workspace of at least nbytes; of at least `least` bytes
-        where nbytes did not fit the device (2D: one step per launch then)."""
+        """The kept workspace of at least nbytes; where nbytes did not fit the
+        device, of at least least(ref) bytes (2D: one step per launch then)."""
         ws = getattr(self, attr)
         if ws is not None and ws.numel() >= nbytes:
             return ws
@@ -363,14 +363,14 @@ class Model:
             try:
                 ws = _workspace(nbytes, self.param.device)
             except torch.OutOfMemoryError:
-                if least >= nbytes:
-                    raise
                 self._denied[attr] = nbytes   # not tried again on every call
             else:
                 setattr(self, attr, ws)
                 return ws
-        if ws is None or ws.numel() < least:
-            setattr(self, attr, _workspace(least, self.param.device))
+        need = _sz(0)
+        _check(least(C.byref(need)), "workspace size")
+        if ws is None or ws.numel() < need.value:
+            setattr(self, attr, _workspace(need.value, self.param.device))
         return getattr(self, attr)
 
     def forward(self, shots: Sequence[Shot], init: Optional[torch.Tensor] = None, return_final: bool = False,
@@ -380,15 +380,15 @@ class Model:
         dev = self.param.device
         traces = [torch.empty((s.nrec, s.nt + 1), dtype=torch.float32, device=dev) for s in shots]
         arr = _shot_descs(shots, traces)
-        nbytes, least = _sz(0), _sz(0)
+        nbytes = _sz(0)
         _check(_fwd_ws(self._h, arr, len(shots), C.byref(nbytes)), "wave_forward_workspace_size")
-        _check(_fwd_min(self._h, arr, len(shots), C.byref(least)), "wave_forward_workspace_min")
         final = torch.empty((2,) + self.shape, dtype=torch.float32, device=dev) if return_final else None
         if init is not None:
             init = init.contiguous().to(torch.float32)
             if tuple(init.shape) != (2,) + self.shape:
                 raise ValueError("init must be [2, *shape]")
-        ws = self._ensure("_fws", nbytes.value, least.value)   # after the outputs: it can do with less
+        # after the outputs: it can do with less
+        ws = self._ensure("_fws", nbytes.value, lambda ref: _fwd_min(self._h, arr, len(shots), ref))
         _check(_forward(self._h, arr, len(shots), _ptr(init), _ptr(final), _ptr(ws), ws.numel(), _stream(stream)),
                "wave_forward")
         return (traces, final) if return_final else traces
@@ -419,14 +419,14 @@ class Model:
         o.k = float(k) if k is not None else 0.0
         o.k_ratio = float(k_ratio) if k_ratio is not None else 0.0
         arr = _shot_descs(shots)
-        nbytes, least = _sz(0), _sz(0)
+        nbytes = _sz(0)
         _check(_grad_ws(self._h, arr, len(shots), C.byref(o), C.byref(nbytes)), "wave_gradient_workspace_size")
-        _check(_grad_min(self._h, arr, len(shots), C.byref(o), C.byref(least)), "wave_gradient_workspace_min")
         grad = out if out is not None else torch.empty(self.shape, dtype=torch.float32, device=dev)
         mis = torch.empty(1, dtype=torch.float64, device=dev)
         kd = torch.empty(1, dtype=torch.float64, device=dev)
         norm = torch.empty(1, dtype=torch.float64, device=dev)
-        ws = self._ensure("_gws", nbytes.value, least.value)   # after the outputs: it can do with less
+        # after the outputs: it can do with less
+        ws = self._ensure("_gws", nbytes.value, lambda ref: _grad_min(self._h, arr, len(shots), C.byref(o), ref))
         _check(_adjoint_sensitivity(self._h, arr, len(shots), C.byref(o), _ptr(grad), _ptr(mis), _ptr(kd),
                                     _ptr(norm), _ptr(ws), ws.numel(), _stream(stream)), "wave_adjoint_sensitivity")
         self.grad_norm = norm
