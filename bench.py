@@ -683,7 +683,8 @@ def main():
                        "storage": args.storage, "parallelism": f"replicas x{world}", "tiling": list(tiling),
                        "cta_order": cta_order,
                        "l2": "inputs larger than L2 (each resident grid > 129 MB)" if 4 * wl.ncells > 129e6
-                       else f"not flushed: grids of {4e-6 * wl.ncells:.2f} MB, which stay in the L2 between steps",
+                       else f"not flushed: levels, coefficients and accumulator of {16e-6 * wl.ncells:.2f} MB, "
+                       + ("larger than L2" if 16 * wl.ncells > 129e6 else "which stay in the L2 between steps"),
                        "observed_data": "true model on a 2x grid with 2x steps" if args.refined_data
                        else "true model on the same grid"},
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clk, "gpu_launches": int(launches),

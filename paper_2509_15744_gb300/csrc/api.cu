@@ -549,7 +549,9 @@ static bool tile2d_pays(const wave_model_s* m, const Tile2DPlan& p, int nfields,
 // A small grid thus takes deep regions (the halo work runs on SMs that would
 // idle), a large one shallow ones.  Measured at the fits' choices and next to
 // them, 251^2 order 2, 6400 steps: 2 rows S = 12 5.1 ms (8: 5.6, 4: 7.6), 4 rows
-// S = 24 6.8; 2048^2 order 8, 800 steps: 4 rows S = 3 16.4 ms (2: 19.1).
+// S = 24 6.8; 2048^2 order 8, 800 steps: 4 rows S = 3 16.4 ms (2: 19.1).  The fits
+// are those of the velocity form with one field; the density form and the
+// two-field modes take them as they are.
 // Grids below 128 cells in x or 16 in y, above 2^32 cells (the second pair of
 // levels costs 2 grids, 34 GB there) and the other storage types keep one step
 // per launch; so do grids that no split fits (order 6 needs h = 12, so fewer than
