@@ -68,8 +68,12 @@ __device__ __forceinline__ void update_store(const StepArgs& a, int64_t off, con
 // ---------------------------------------------------------------------------
 // 2D: warp-per-strip, march in y
 // ---------------------------------------------------------------------------
+// 16-bit storage is held to the CTAs per SM that its default split counts on:
+// seven at order 4 (72 registers; ptxas takes 76 by itself, the last CTAs of a
+// launch of about 6 per SM then run alone: 4096^2, BF16, a gradient of 12 steps 3.7
+// ms, 2.5 held) and five at order 8 (96 instead of 98).
 template <int R, typename T, int WPB>
-__global__ void __launch_bounds__(WPB * 32)
+__global__ void __launch_bounds__(WPB * 32, sizeof(T) == 2 && R == 2 ? 7 : sizeof(T) == 2 && R == 4 ? 5 : 0)
 step2d_velocity_kernel(StepArgs a) {
   __shared__ __align__(16) float sm[WPB][kRowW];
   chain_wait();
@@ -78,8 +82,8 @@ step2d_velocity_kernel(StepArgs a) {
   const int warp = threadIdx.x >> 5;
   const int64_t nstrips = (g.nx + kStrip - 1) / kStrip;
   const int64_t gw = (int64_t)blockIdx.x * WPB + warp;
-  const int64_t strip = gw % nstrips;
-  const int64_t y0 = (gw / nstrips) * a.zblock;
+  const int64_t yb = gw / nstrips, strip = gw - yb * nstrips;
+  const int64_t y0 = yb * a.zblock;
   if (y0 >= g.ny) return;  // warp-uniform; this kernel synchronises only within warps
   const int64_t y1 = min(y0 + a.zblock, g.ny);
   const int64_t x0 = strip * kStrip;
