@@ -251,6 +251,16 @@ static cudaError_t launch_vel(const StepArgs& a, cudaStream_t s) {
     const int64_t warps = nstrips * nyb;
     const int64_t blocks = (warps + kWarps2D - 1) / kWarps2D;
     count_launch();
+    if constexpr (sizeof(T) == 2 && R <= 2) {
+      // long marches suffer from the uneven placement of chained CTAs (as in 3D
+      // below) more than they gain from the earlier start: BF16, order 2, 12 steps
+      // of 30000 x 100 (8 rows a warp) 0.55 ms chained, 0.51 plain; 1024^2 (2 rows)
+      // 0.30 and 0.33
+      if (a.zblock >= 8) {
+        step2d_velocity_kernel<R, T, kWarps2D><<<(unsigned)blocks, kWarps2D * 32, 0, s>>>(a);
+        return cudaGetLastError();
+      }
+    }
     return launch_chained(step2d_velocity_kernel<R, T, kWarps2D>, (unsigned)blocks, kWarps2D * 32, 0, s, a);
   } else {
     dim3 grid((unsigned)nstrips, (unsigned)((g.ny + kRows3D - 1) / kRows3D),
