@@ -254,8 +254,10 @@ step3d_velocity_pair_kernel(BatchArgs b) {
     auto stage = [&](int p, int buf) {
       // Most planes of most CTAs mirror nothing: copies from a running pointer,
       // without the masks (512^3 x 8 shots 3068 -> 3020 us a launch, 1024^3 x 4
-      // with compensation 14.79 -> 14.25 ms).
-      if (yplain && p < nz_plain) {
+      // with compensation 14.79 -> 14.25 ms).  Not at orders 4 and 6 with the
+      // accumulator in tensor memory, whose code comes out slower for it (256^3 x 8,
+      // 10 steps, a gradient: order 6 13.7 ms, 12.4 without; order 4 12.1 and 11.8).
+      if (!((R == 2 || R == 3) && TM && ACC == kPairSq) && yplain && p < nz_plain) {
         const uint32_t sb = smem0 + (uint32_t)(buf * PT::TILE) * 4u;
         constexpr uint32_t fB = (uint32_t)(NB * PT::TILE) * 4u;
         pcp16(sb + d0, sA + c_off[0], c_sz[0]);
