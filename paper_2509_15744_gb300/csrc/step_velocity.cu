@@ -269,10 +269,12 @@ static cudaError_t launch_vel(const StepArgs& a, cudaStream_t s) {
       return launch_step3d_ring(a, 2 * R, s);
     } else {
       count_launch();
-      // more full z-blocks than two CTAs per SM take at once (the last block of a
-      // column counts by its planes: 33 x 500 x 384, order 8, 378 CTAs of which
-      // half have one plane, takes 1.40 ms by itself and 1.80 held)
-      if (R >= 3 && (int64_t)grid.x * grid.y * g.nz > 2 * 152 * a.zblock)
+      // more z-blocks than two CTAs per SM take at once, a last one counted from three
+      // quarters of the planes on (33 x 500 x 384, order 8, 378 CTAs of which half
+      // have one plane: 1.40 ms by itself and 1.80 held; six steps of 49 x 400 x 500,
+      // 200 CTAs of 32 planes and 200 of 17: 0.39 and 0.46)
+      const int64_t blocks = (int64_t)grid.x * grid.y * ((g.nz + a.zblock / 4) / a.zblock);
+      if (R >= 3 && blocks > 2 * 152)
         step3d_velocity_kernel<R, T, kRows3D, R >= 3 ? 4 : 0><<<grid, kRows3D * 32, 0, s>>>(a);
       else
         step3d_velocity_kernel<R, T, kRows3D, 0><<<grid, kRows3D * 32, 0, s>>>(a);
